@@ -130,8 +130,8 @@ def run_mlp(args, B, torch):
     """Throughput of the wall model's network on its tcgen05 kernels: inference
     (the fused kernel: 180 B of input and output per row for 110 kFLOP, so bound by
     the tensor cores and the on-chip epilogues, not by HBM) and the training step
-    (layer by layer: every z is stored for the backward pass, 64 FLOPs per byte at
-    the 128-wide layers, so HBM-bound) on 65,536 rows (the training batch; a
+    (forward, loss and data gradients of a 128-row tile on chip, the BF16 operands
+    of the weight gradients through global memory) on 65,536 rows (the training batch; a
     coupled step of the 128x49x128 grid feeds 32,768)."""
     import ctypes as C
 
@@ -169,9 +169,9 @@ def run_mlp(args, B, torch):
     flops_f = 2.0 * rows * macs
     # the fused inference kernel reads each input row and writes its outputs, nothing else
     bytes_f = 4.0 * rows * (40 + 5)
-    # the training step's forward stores every layer's z for the backward pass: FP32 values
-    # read + written per row: input scaling 40 + 40, layers (40 + 128) + 3 (128 + 128) + (128 + 5)
-    bytes_train_fwd = 4.0 * rows * (80 + 168 + 3 * 256 + 133)
+    # the training step reads inputs and labels (FP32) and writes, then reads, the BF16 operand
+    # tiles of the weight gradients: activations 48 + 4 x 128, output gradients 4 x 128 + 16
+    bytes_train = rows * (4.0 * 45 + 2 * 2.0 * (48 + 8 * 128 + 16))
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
@@ -187,7 +187,7 @@ def run_mlp(args, B, torch):
                                 "per_unit": f"2 x {macs} FLOPs per row x {rows} rows (180 B per row: "
                                             f"{bytes_f / t_f / 1e9:.0f} GB/s, {bytes_f / t_f / 1e9 / hbm:.3f} of HBM)",
                                 "peak_source": "MEASURED_PEAKS.json bf16_tflops (cuBLAS burst)"},
-           "train_step_forward_bytes_per_row": bytes_train_fwd / rows, "status": net.status()}
+           "train_step_bytes_per_row": bytes_train / rows, "status": net.status()}
     net.close()
     return out
 

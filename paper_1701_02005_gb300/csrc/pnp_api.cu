@@ -2297,12 +2297,9 @@ void pnp_ensemble_destroy(pnp_ensemble* e) {
 // ---------------------------------------------------------------------------
 // Learned wall model: MLP workspace and the coupling to a coarse context.
 // ---------------------------------------------------------------------------
-constexpr int kMlpMaxPartial = 320;
-
 struct pnp_mlp {
   MlpBufs b{};
   int max_batch = 0;
-  int max_partial = 64;   // weight-gradient CTAs: two per SM (at most kMlpMaxPartial)
   size_t nparam = 0;
   cudaStream_t stream = nullptr;
   int t_adam = 0;
@@ -2313,19 +2310,19 @@ namespace {
 size_t mlp_carve(pnp_mlp* m, char* base, int max_batch) {
   Bump bp{base};
   const MlpDims d = mlp_dims();
-  const size_t np = d.nparam, B = (size_t)max_batch;
+  const size_t np = d.nparam;
   MlpBufs b{};
   b.param = bp.take<float>(np);
-  b.wimg = bp.take<__nv_bfloat16>(mlp_images().total);
+  b.wimg = bp.take<__nv_bfloat16>(mlp_image_elems());
   b.grad = bp.take<float>(np);
   b.m = bp.take<float>(np);
   b.v = bp.take<float>(np);
-  b.act[0] = bp.take<float>(B * kMlpIn);
-  for (int l = 0; l < kMlpLayers; ++l) b.act[l + 1] = bp.take<float>(B * d.out[l]);
-  b.dact = bp.take<float>(B * kMlpHidden);
-  b.dact2 = bp.take<float>(B * kMlpHidden);
-  b.partial = bp.take<float>(kMlpMaxPartial * (size_t)(kMlpHidden * kMlpHidden + kMlpHidden));
-  b.loss = bp.take<float>(128);
+  const int ntiles = (max_batch - 1) / 128 + 1;
+  b.atiles = bp.take<unsigned char>(ntiles * kATileBytes);
+  b.dztiles = bp.take<unsigned char>(ntiles * kDzTileBytes);
+  b.partial = bp.take<float>(mlp_wgrad_plan(ntiles).total);
+  b.lpart = bp.take<float>(8 * kMlpMaxRowCtas);
+  b.loss = bp.take<float>(1);
   b.in_shift = bp.take<float>(kMlpIn);
   b.in_scale = bp.take<float>(kMlpIn);
   b.out_shift = bp.take<float>(kMlpOut);
@@ -2381,12 +2378,6 @@ int pnp_mlp_create(pnp_mlp** out, int max_batch, void* ws, size_t bytes, void* s
   if (!m) return PNP_ERR_ARG;
   m->max_batch = max_batch;
   m->stream = (cudaStream_t)stream;
-  {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
-      m->max_partial = std::min(2 * sms, kMlpMaxPartial);
-  }
   mlp_carve(m, (char*)ws, max_batch);
   // weights U(-a, a), a = sqrt(6 / fan_in) from SplitMix64; biases 0; unit normalisation
   const MlpDims d = mlp_dims();
@@ -2403,7 +2394,7 @@ int pnp_mlp_create(pnp_mlp** out, int max_batch, void* ws, size_t bytes, void* s
   ok = ok && cudaMemcpyAsync(m->b.param, p.data(), sizeof(float) * d.nparam, cudaMemcpyHostToDevice, m->stream) == cudaSuccess;
   ok = ok && cudaMemcpyAsync(m->b.in_scale, ones.data(), sizeof(float) * kMlpIn, cudaMemcpyHostToDevice, m->stream) == cudaSuccess;
   ok = ok && cudaMemcpyAsync(m->b.out_scale, ones.data(), sizeof(float) * kMlpOut, cudaMemcpyHostToDevice, m->stream) == cudaSuccess;
-  ok = ok && mlp_sync_bf16(m->b, d.nparam, m->stream) == cudaSuccess;
+  ok = ok && mlp_make_images(m->b.param, m->b.wimg, m->stream) == cudaSuccess;
   ok = ok && cudaStreamSynchronize(m->stream) == cudaSuccess;
   if (!ok) { delete m; return PNP_ERR_CUDA; }
   *out = m;
@@ -2422,7 +2413,7 @@ int pnp_mlp_set_params(pnp_mlp* m, const float* host, size_t n) {
   CK(cudaMemcpyAsync(m->b.param, host, sizeof(float) * n, cudaMemcpyHostToDevice, m->stream));
   CK(cudaMemsetAsync(m->b.m, 0, sizeof(float) * n, m->stream));
   CK(cudaMemsetAsync(m->b.v, 0, sizeof(float) * n, m->stream));
-  CK(mlp_sync_bf16(m->b, n, m->stream));
+  CK(mlp_make_images(m->b.param, m->b.wimg, m->stream));
   CK(cudaStreamSynchronize(m->stream));
   m->t_adam = 0;
   return PNP_OK;
@@ -2448,28 +2439,26 @@ int pnp_mlp_set_skip(pnp_mlp* m, int out_col, int in_col) {
 
 int pnp_mlp_forward(pnp_mlp* m, const float* X, int B, float* Y) {
   if (!m || !X || !Y || B < 1 || B > m->max_batch) return PNP_ERR_ARG;
-  CK(mlp_forward(m->b, X, B, Y, m->stream));
+  CK(mlp_infer_tc(m->b, X, B, Y, m->stream));
   return PNP_OK;
 }
 
 int pnp_mlp_gradient(pnp_mlp* m, const float* X, const float* T, int B, float* grad_host, float* loss_host) {
   if (!m || !X || !T || B < 1 || B > m->max_batch) return PNP_ERR_ARG;
-  CK(mlp_forward(m->b, X, B, nullptr, m->stream));
-  CK(mlp_backward(m->b, X, T, B, m->max_partial, m->stream));
+  CK(mlp_train_tc(m->b, X, T, B, m->stream));
   if (grad_host) CK(cudaMemcpyAsync(grad_host, m->b.grad, sizeof(float) * m->nparam, cudaMemcpyDeviceToHost, m->stream));
-  if (loss_host) CK(cudaMemcpyAsync(loss_host, m->b.loss + 120, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
+  if (loss_host) CK(cudaMemcpyAsync(loss_host, m->b.loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
   CK(cudaStreamSynchronize(m->stream));
   return PNP_OK;
 }
 
 int pnp_mlp_train_step(pnp_mlp* m, const float* X, const float* T, int B, float lr, float* loss_host) {
   if (!m || !X || !T || B < 1 || B > m->max_batch || !(lr > 0)) return PNP_ERR_ARG;
-  CK(mlp_forward(m->b, X, B, nullptr, m->stream));
-  CK(mlp_backward(m->b, X, T, B, m->max_partial, m->stream));
+  CK(mlp_train_tc(m->b, X, T, B, m->stream));
   m->t_adam += 1;
   CK(mlp_adam(m->b, m->nparam, lr, 0.9f, 0.999f, 1e-8f, m->t_adam, m->stream));
   if (loss_host) {
-    CK(cudaMemcpyAsync(loss_host, m->b.loss + 120, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
+    CK(cudaMemcpyAsync(loss_host, m->b.loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
   }
   return PNP_OK;
@@ -2705,7 +2694,7 @@ int pnp_step_wallmodel(pnp_ctx* c, pnp_mlp* m, int nsteps, double dt) {
   for (int n = 0; n < nsteps; ++n) {
     int r = pnp_wall_features(c, 8, c->featX);
     if (r) return r;
-    CK(mlp_forward(m->b, c->featX, rows, c->featY, c->stream));
+    CK(mlp_infer_tc(m->b, c->featX, rows, c->featY, c->stream));
     if (c->wm_mode == 2) CK(launch_mean_rates(c->featY, rows / 2, c->stream));
     if (c->wm_mode <= 2) {   // mode 3 leaves the wall shear to the solver's own no-slip walls
       if (c->wm_relax < 1.f) {   // the rates used move a fraction of the way to the prediction

@@ -75,49 +75,43 @@ struct MlpDims {
 };
 MlpDims mlp_dims();
 
-// Offsets (BF16 elements) of the weight images: per layer the forward GEMM's B
-// tile [Np][Kp] and the data gradient's [Kp][Np], in the shared-memory layout.
-struct MlpImg {
-  size_t fwd[kMlpLayers], bwd[kMlpLayers];
-  size_t total;
-};
-MlpImg mlp_images();
+size_t mlp_image_elems();   // BF16 elements of the weight images
 cudaError_t mlp_make_images(const float* param, __nv_bfloat16* img, cudaStream_t s);
+
+// Operand tiles of 128 rows that the training kernel leaves for the weight
+// gradients: a_0 [128][48], a_1 .. a_4 [128][128]; dz_1 .. dz_4 [128][128], dz_5 [128][16].
+constexpr int kTileBytes = 128 * kMlpHidden * 2, kA0Bytes = 128 * 48 * 2;
+constexpr size_t kATileBytes = kA0Bytes + 4 * (size_t)kTileBytes, kDzTileBytes = 4 * (size_t)kTileBytes + 128 * 16 * 2;
+constexpr int kMlpMaxRowCtas = 512;   // CTAs of the training kernel (partial losses)
+
+// CTAs per layer of the weight gradients, and the layers' slices of the partial sums.
+struct WgPlan {
+  int splits[kMlpLayers];
+  size_t len[kMlpLayers], off[kMlpLayers], total;
+};
+WgPlan mlp_wgrad_plan(int ntiles);
 
 // Buffers of one MLP (all device pointers, carved by the host code).
 struct MlpBufs {
   float* param;        // FP32 master weights and biases
-  __nv_bfloat16* wimg; // BF16 weight images of the GEMMs (mlp_images), rebuilt from param
+  __nv_bfloat16* wimg; // BF16 weight images of the GEMMs, rebuilt from param
   float* grad;         // gradient of the loss
   float* m;            // Adam first moment
   float* v;            // Adam second moment
-  float* act[kMlpLayers + 1];   // act[0] normalised input, act[l+1] output of layer l (pre-activation z)
-  float* dact;         // backward scratch [B][128]
-  float* dact2;        // backward scratch [B][128]
-  float* partial;      // per-block partial weight gradients
-  float* loss;         // [partial blocks] then the reduced loss
+  unsigned char *atiles, *dztiles;   // operand tiles, kATileBytes / kDzTileBytes per 128 rows
+  float* partial;      // per-CTA partial weight gradients
+  float* lpart;        // [row CTAs][8] squared errors and output-bias gradients
+  float* loss;         // the reduced loss
   float *in_shift, *in_scale, *out_shift, *out_scale;
   int* err;            // device status word (PNP_ERR_TIMEOUT from a bounded tensor-core wait)
   int skip_out = -1;   // residual output: y[skip_out] = network + x[skip_in] (none when < 0)
   int skip_in = -1;
 };
 
-// Tensor-core (tcgen05) GEMMs of the MLP (k_mlp_tc.cu).
-cudaError_t mlp_fwd_layer_tc(const float* in, int K, bool act_in, const __nv_bfloat16* Wimg, const float* bias, int N,
-                             int B, float* out, int* err, cudaStream_t s);
-cudaError_t mlp_bwd_data_tc(const float* dz, int N, const __nv_bfloat16* WimgT, int K, int B, const float* zprev,
-                            float* out, int* err, cudaStream_t s);
-cudaError_t mlp_wgrad_tc(const float* dz, int N, const float* in, int K, bool act_in, int B, int rows_per_block,
-                         int nblk, float* partial, int* err, cudaStream_t s);
-
-// The whole network in one persistent kernel, outputs only (inference).
-cudaError_t mlp_infer_tc(const float* X, int B, const __nv_bfloat16* wimg, const float* param,
-                         const float* in_shift, const float* in_scale, const float* out_shift, const float* out_scale,
-                         int skip_out, int skip_in, float* Y, int* err, cudaStream_t s);
-
-cudaError_t mlp_sync_bf16(const MlpBufs& b, size_t nparam, cudaStream_t s);
-cudaError_t mlp_forward(const MlpBufs& b, const float* X, int B, float* Y, cudaStream_t s);
-cudaError_t mlp_backward(const MlpBufs& b, const float* X, const float* T, int B, int max_partial, cudaStream_t s);
+// The network on the tensor cores (k_mlp_tc.cu): outputs only, or the gradient
+// of the loss into b.grad and the loss into b.loss.
+cudaError_t mlp_infer_tc(const MlpBufs& b, const float* X, int B, float* Y, cudaStream_t s);
+cudaError_t mlp_train_tc(const MlpBufs& b, const float* X, const float* T, int B, cudaStream_t s);
 cudaError_t mlp_adam(const MlpBufs& b, size_t nparam, float lr, float beta1, float beta2, float eps, int t,
                      cudaStream_t s);
 
