@@ -348,7 +348,8 @@ int pnp_fp64_peak(pnp_ctx* ctx, double* flops_out);
  * 32 / 64 cells wide, 128 TMA rows), the
  * wall-normal CN sweeps (32 = mixed
  * shared-memory line tiles, else 64/128/256 threads per block), the spectral
- * y-solves (16 = mixed shared-memory tiles, else 32/64/128 threads) and the
+ * y-solves (mixed: 16 = columns in shared memory, 32 = streamed; other codes
+ * choose by the grid) and the
  * z-transform (8..64 threads per column; mixed: 64 = stage-by-stage kernel,
  * else register FFT) on this context's grid with CUDA events and keeps the
  * fastest; then re-checks each choice, one code at a time, on the time of

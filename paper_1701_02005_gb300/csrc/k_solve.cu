@@ -737,13 +737,16 @@ cudaError_t launch_fft_z(cplx<T>* spec, const cplx<T>* tw_z, const Geo& g, bool 
 }
 
 // ---------------------------------------------------------------------------
-// Spectral Thomas: per (m, n), solve a_j x_{j-1} + (b_j - kx2_m - kz2_n) x_j
-// + c_j x_{j+1} = scale * rhs_j in FP64.  The Neumann (0,0) mode replaces its
-// bottom-row equation by x_0 = 0.  The elimination factors depend only on the
-// grid, so they are computed once (k_spec_factors): inv_j = 1 / (B_j - a_j
-// c'_{j-1}) and c'_j = c_j inv_j, stored per spectral point in FP64.
-// The sweeps load CH planes ahead so that a thread keeps CH independent
-// memory requests in flight instead of one per serial step.
+// Spectral y-solves: per (m, n), a_j x_{j-1} + (b_j - kx2_m - kz2_n) x_j + c_j
+// x_{j+1} = scale * rhs_j, with the Neumann (0,0) mode's bottom-row equation
+// replaced by x_0 = 0.  The elimination runs from both walls at once and meets at
+// the middle row tw = n / 2 (a twisted factorisation):
+//   below  d_j = (r_j - a_j d_{j-1}) inv_j,  x_j = d_j - cpr_j x_{j+1}, cpr_j = c_j inv_j
+//   above  d_j = (r_j - c_j d_{j+1}) inv_j,  x_j = d_j - cpr_j x_{j-1}, cpr_j = a_j inv_j
+//   x_tw = (r_tw - a_tw d_{tw-1} - c_tw d_{tw+1}) inv_tw
+// with inv_tw the pivot of row tw after both eliminations: as many operations as
+// one elimination through the column, as two independent chains of half the
+// length.  The factors depend only on the grid and are computed once, in FP64.
 // ---------------------------------------------------------------------------
 __global__ void k_spec_factors(double* __restrict__ cpr, double* __restrict__ inv, const double* __restrict__ kx2,
                                const double* __restrict__ kz2, YRows rows, Geo g, bool neumann) {
@@ -754,15 +757,25 @@ __global__ void k_spec_factors(double* __restrict__ cpr, double* __restrict__ in
   const size_t base = (size_t)n * g.mp + mm;
   const double k2 = kx2[mm] + kz2[n];
   const bool pin = neumann && mm == 0 && n == 0;
-  double cprev = 0.0;
-  for (int j = 0; j < g.nyc; ++j) {
+  const int tw = g.nyc / 2;
+  double lo = 0.0, hi = 0.0;   // cpr of the row before, from below and from above
+  for (int j = 0; j < tw; ++j) {
     double a = rows.a[j], b = rows.b[j] - k2, c = rows.c[j];
     if (pin && j == 0) { b = 1.0; c = 0.0; }
-    const double iv = 1.0 / (b - a * cprev);
-    cprev = c * iv;
-    cpr[base + (size_t)j * P] = cprev;
+    const double iv = 1.0 / (b - a * lo);
+    lo = c * iv;
+    cpr[base + (size_t)j * P] = lo;
     inv[base + (size_t)j * P] = iv;
   }
+  for (int j = g.nyc - 1; j > tw; --j) {
+    const double a = rows.a[j], b = rows.b[j] - k2, c = rows.c[j];
+    const double iv = 1.0 / (b - c * hi);
+    hi = a * iv;
+    cpr[base + (size_t)j * P] = hi;
+    inv[base + (size_t)j * P] = iv;
+  }
+  cpr[base + (size_t)tw * P] = 0.0;
+  inv[base + (size_t)tw * P] = 1.0 / (rows.b[tw] - k2 - rows.a[tw] * lo - rows.c[tw] * hi);
 }
 
 cudaError_t launch_spec_factors(double* cpr, double* inv, const double* kx2, const double* kz2, const YRows& rows,
@@ -773,250 +786,375 @@ cudaError_t launch_spec_factors(double* cpr, double* inv, const double* kx2, con
   return cudaGetLastError();
 }
 
-constexpr int kCH = 8;
-
-// FP64 (0,0) mode of the mixed potential: the FP32 transform's mean of the
-// fluctuating charge, scaled, plus the FP64 reference source; the solution goes
-// to mean_out (plus mean_shift) and the transform slot is zeroed.  Runs in the
-// real-part thread; the imaginary-part thread only zeroes its slots.
-template <typename T>
-__device__ void spec_mean_mode(T* sp, const double* __restrict__ cpr, const double* __restrict__ inv,
-                               const YRows& rows, size_t base, size_t P, int ny, int part, double scale,
-                               const double* __restrict__ mean_rhs, const double* __restrict__ mean_shift,
-                               double* __restrict__ mean_out) {
-  if (part == 1) {
-    for (int j = 0; j < ny; ++j) sp[2 * (base + (size_t)j * P)] = T(0);
-    return;
-  }
-  double d = 0.0;
-  for (int j0 = 0; j0 < ny; j0 += kCH) {
-    double rr[kCH], iv[kCH], mr[kCH];
-#pragma unroll
-    for (int u = 0; u < kCH; ++u)
-      if (j0 + u < ny) {
-        const size_t o = base + (size_t)(j0 + u) * P;
-        rr[u] = (double)sp[2 * o];
-        iv[u] = inv[o];
-        mr[u] = mean_rhs[j0 + u];
-      }
-#pragma unroll
-    for (int u = 0; u < kCH; ++u)
-      if (j0 + u < ny) {
-        d = (rr[u] * scale + mr[u] - rows.a[j0 + u] * d) * iv[u];
-        mean_out[j0 + u] = d;
-      }
-  }
-  double x = d;
-  mean_out[ny - 1] = x + mean_shift[ny - 1];
-  sp[2 * (base + (size_t)(ny - 1) * P)] = T(0);
-  for (int j1 = ny - 2; j1 >= 0; j1 -= kCH) {
-    double dd[kCH], cc[kCH], ms[kCH];
-#pragma unroll
-    for (int u = 0; u < kCH; ++u)
-      if (j1 - u >= 0) {
-        dd[u] = mean_out[j1 - u];
-        cc[u] = cpr[base + (size_t)(j1 - u) * P];
-        ms[u] = mean_shift[j1 - u];
-      }
-#pragma unroll
-    for (int u = 0; u < kCH; ++u)
-      if (j1 - u >= 0) {
-        x = dd[u] - cc[u] * x;
-        mean_out[j1 - u] = x + ms[u];
-        sp[2 * (base + (size_t)(j1 - u) * P)] = T(0);
-      }
+// Mixed path: the recurrences run in double-float on the FP32 pipe (pnp_df.cuh).
+// The low wavenumbers are ill-conditioned on the stretched grid (the near-wall
+// rows dominate |A| |x| by orders of magnitude over A x), so they need more than
+// FP32; df carries a 48-bit significand at a small fraction of the FP64 pipe time.
+__device__ __forceinline__ void sp_cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void sp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void sp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// all but the groups after number g of four, then one more
+__device__ __forceinline__ void sp_wait_group(int g) {
+  switch (g) {
+    case 0: sp_wait<4>(); break;
+    case 1: sp_wait<3>(); break;
+    case 2: sp_wait<2>(); break;
+    default: sp_wait<1>(); break;
   }
 }
+constexpr int kSpRows = 4;   // rows per batch of loads
 
-// The forward sweep runs on the unscaled transform; its FP64 results go to an
-// FP64 scratch (no round trip through the transform's precision), and the
-// normalisation 1/(Nx Nz) is applied once, in the transform's precision, when
-// the solution is stored.  The real and imaginary parts are independent
-// recurrences with the same coefficients, so each runs in its own thread
-// (adjacent threads touch the two halves of one complex value).  The FP64 mean
-// mode (mixed potential) keeps the scaled physical source and never touches
-// spec; it runs in the real-part thread of (0,0).
-template <typename T>
-__global__ void k_spec_thomas(cplx<T>* __restrict__ spec, cplx<double>* __restrict__ dscr,
-                              const double* __restrict__ cpr, const double* __restrict__ inv, YRows rows, Geo g,
-                              double scale, bool neumann, const double* __restrict__ mean_rhs,
-                              const double* __restrict__ mean_shift, double* __restrict__ mean_out) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int mm = tid >> 1, part = tid & 1;
-  const int n = blockIdx.y;
-  if (mm >= g.mh) return;
-  const size_t P = (size_t)g.nz * g.mp;
-  const size_t base = (size_t)n * g.mp + mm;
-  const int ny = g.nyc;
-  T* sp = reinterpret_cast<T*>(spec) + part;             // this part of spec[base + j P] at sp[2 (base + j P)]
-  double* dp = reinterpret_cast<double*>(dscr) + part;
-  const bool pin = neumann && mm == 0 && n == 0;
-  const bool mean_mode = mean_rhs != nullptr && mm == 0 && n == 0;
-  if (mean_mode) {
-    spec_mean_mode(sp, cpr, inv, rows, base, P, ny, part, scale, mean_rhs, mean_shift, mean_out);
-    return;
-  }
-  double d = 0.0;
-  for (int j0 = 0; j0 < ny; j0 += kCH) {
-    double rr[kCH], iv[kCH];
-#pragma unroll
-    for (int u = 0; u < kCH; ++u) {
-      if (j0 + u < ny) {
-        const size_t o = base + (size_t)(j0 + u) * P;
-        rr[u] = (double)sp[2 * o];
-        iv[u] = inv[o];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kCH; ++u) {
-      const int j = j0 + u;
-      if (j < ny) {
-        const double r = (pin && j == 0) ? 0.0 : rr[u];
-        d = (r - rows.a[j] * d) * iv[u];
-        dp[2 * (base + (size_t)j * P)] = d;
-      }
-    }
-  }
-  const T sc = (T)scale;
-  double x = d;
-  sp[2 * (base + (size_t)(ny - 1) * P)] = (T)x * sc;
-  for (int j1 = ny - 2; j1 >= 0; j1 -= kCH) {
-    double dd[kCH], cc[kCH];
-#pragma unroll
-    for (int u = 0; u < kCH; ++u) {
-      if (j1 - u >= 0) {
-        const size_t o = base + (size_t)(j1 - u) * P;
-        dd[u] = dp[2 * o];
-        cc[u] = cpr[o];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kCH; ++u) {
-      const int j = j1 - u;
-      if (j >= 0) {
-        x = dd[u] - cc[u] * x;
-        sp[2 * (base + (size_t)j * P)] = (T)x * sc;
-      }
-    }
-  }
+// Rows per copy group of a sweep over `rows` rows, a multiple of the batch.
+__device__ __forceinline__ int sp_group_rows(int rows) {
+  return max(kSpRows, ((rows + 3) / 4 + kSpRows - 1) / kSpRows * kSpRows);
 }
 
-template <typename T>
-cudaError_t launch_spec_thomas(cplx<T>* spec, cplx<double>* dscr, const double* cpr, const double* inv,
-                               const YRows& rows, const Geo& g, double scale, bool neumann, cudaStream_t s,
-                               const double* mean_rhs, const double* mean_shift, double* mean_out) {
-  const int T_ = g.lc_spec ? g.lc_spec : 64;
-  dim3 grd((2 * g.mh + T_ - 1) / T_, g.nz, 1);
-  k_spec_thomas<T><<<grd, T_, 0, s>>>(spec, dscr, cpr, inv, rows, g, scale, neumann, mean_rhs, mean_shift, mean_out);
-  return cudaGetLastError();
-}
+// Per row of 16 points: transform values, 1/pivot, cpr, and the two off-diagonals.
+constexpr size_t spec_smem_df(int n) { return (size_t)n * (3 * 16 * 8 + 2 * 8); }
 
-// Rows per batch of the df line sweeps (two batches in flight per thread).
-constexpr int kDfCH = 4;
-
-// Mixed path: the same elimination in double-float arithmetic on the FP32 pipe
-// (pnp_df.cuh).  The low wavenumbers are ill-conditioned on the stretched grid
-// (the near-wall rows dominate |A| |x| by orders of magnitude over A x), so the
-// recurrence needs more than FP32; df carries a 48-bit significand at a small
-// fraction of the FP64 pipe time.  Factors c'_j, 1/pivot_j and the
-// sub-diagonal a_j arrive as df pairs (converted once from the FP64 factors);
-// the forward-sweep values go to the scratch as df pairs; the (0,0) mode of the
-// mixed potential keeps its FP64 path.
-__global__ void k_spec_thomas_df(cplx<float>* __restrict__ spec, float2* __restrict__ dscr,
-                                 const float2* __restrict__ cprF, const float2* __restrict__ invF,
-                                 const float2* __restrict__ aF, const double* __restrict__ cpr,
-                                 const double* __restrict__ inv, YRows rows, Geo g, double scale, float sc,
-                                 bool neumann, const double* __restrict__ mean_rhs,
-                                 const double* __restrict__ mean_shift, double* __restrict__ mean_out) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int mm = tid >> 1, part = tid & 1;
-  const int n = blockIdx.y;
-  if (mm >= g.mh) return;
-  const size_t P = (size_t)g.nz * g.mp;
-  const size_t base = (size_t)n * g.mp + mm;
-  const int ny = g.nyc;
-  float* sp = reinterpret_cast<float*>(spec) + part;   // this part of spec[base + j P] at sp[2 (base + j P)]
-  float2* dp = dscr + part;                             // its df forward value at dp[2 (base + j P)]
-  const bool pin = neumann && mm == 0 && n == 0;
-  if (mean_rhs != nullptr && mm == 0 && n == 0) return;   // k_spec_mean handles the (0,0) mode
-  // Both sweeps run in kDfCH-row batches, double-buffered: the loads of batch
-  // b + 1 are in flight while batch b's recurrence runs.
-  auto load_f = [&](int j0, float (&rr)[kDfCH], float2 (&iv)[kDfCH]) {
-#pragma unroll
-    for (int u = 0; u < kDfCH; ++u)
-      if (j0 + u < ny) {
-        const size_t o = base + (size_t)(j0 + u) * P;
-        rr[u] = sp[2 * o];
-        iv[u] = invF[o];
-      }
-  };
-  auto comp_f = [&](int j0, const float (&rr)[kDfCH], const float2 (&iv)[kDfCH], dfl d) {
-#pragma unroll
-    for (int u = 0; u < kDfCH; ++u) {
-      const int j = j0 + u;
-      if (j < ny) {
-        const float r = (pin && j == 0) ? 0.f : rr[u];
-        const float2 a = aF[j];
-        d = df_mul(df_sub_mul(r, dfl{a.x, a.y}, d), dfl{iv[u].x, iv[u].y});
-        if (j < ny - 1) dp[2 * (base + (size_t)j * P)] = make_float2(d.h, d.l);
-      }
-    }
-    return d;
-  };
-  dfl d{0.f, 0.f};
+// Columns in shared memory, double-float.  A warp solves 16 consecutive spectral
+// points of the plane (n mp + m, padding columns included), both parts of a point
+// in one lane (packed FP32): lanes 0-15 eliminate from the bottom wall, lanes
+// 16-31 from the top wall.  Every load of the block is issued before the first
+// operation (cp.async: four groups of rows in sweep order and one for the back
+// substitution's factors), so a column costs one memory latency instead of one
+// per batch of rows, and the forward values make no round trip: they replace the
+// transform value (leading parts) and 1/pivot (trailing parts) of their row.
+__global__ void __launch_bounds__(32)
+    k_spec_df_smem(cplx<float>* __restrict__ spec, SpecDF f, Geo g, float sc, bool neumann, bool skip_mean) {
+  extern __shared__ __align__(16) unsigned char sp_smem[];
+  const int n = g.nyc, tw = n / 2;
+  float2* rr = reinterpret_cast<float2*>(sp_smem);   // [n][16]
+  float2* iv = rr + (size_t)n * 16;                  // [n][16]
+  float2* cc = iv + (size_t)n * 16;                  // [n][16]
+  float2* ee = cc + (size_t)n * 16;                  // [2][n]: a, c
+  const int t = threadIdx.x, half = t >> 4, q = t & 15;
+  const size_t P = (size_t)g.nz * g.mp, p0 = (size_t)blockIdx.x * 16;
+  const int most = max(tw, n - 1 - tw);              // rows of the longer sweep (the upper one: one more at most)
+  const int per = sp_group_rows(most);
   {
-    float rA[kDfCH], rB[kDfCH];
-    float2 iA[kDfCH], iB[kDfCH];
-    load_f(0, rA, iA);
-    for (int j0 = 0; j0 < ny; j0 += 2 * kDfCH) {
-      if (j0 + kDfCH < ny) load_f(j0 + kDfCH, rB, iB);
-      d = comp_f(j0, rA, iA, d);
-      if (j0 + kDfCH < ny) {
-        if (j0 + 2 * kDfCH < ny) load_f(j0 + 2 * kDfCH, rA, iA);
-        d = comp_f(j0 + kDfCH, rB, iB, d);
+    // copy e of a pair of rows (step i of both sweeps): 8 16-byte copies per row and array
+    const int c = t & 7, h = (t >> 3) & 1, arr = t >> 4;
+    const char* src = arr ? reinterpret_cast<const char*>(f.inv + p0) : reinterpret_cast<const char*>(spec + p0);
+    char* dst = reinterpret_cast<char*>(arr ? iv : rr);
+    for (int gr = 0; gr < 4; ++gr) {
+      const int i1 = min(most, (gr + 1) * per);
+      for (int i = gr * per; i < i1; ++i) {
+        const int j = h ? n - 1 - i : i;
+        if (h ? j > tw : j < tw) sp_cp_async16(dst + (size_t)j * 128 + 16 * c, src + (size_t)j * P * 8 + 16 * c);
       }
+      if (gr == 3 && h == 0) sp_cp_async16(dst + (size_t)tw * 128 + 16 * c, src + (size_t)tw * P * 8 + 16 * c);
+      sp_commit();
     }
+    const char* cs = reinterpret_cast<const char*>(f.cpr + p0);
+    for (int i = most - 1 - arr; i >= 0; i -= 2) {   // two steps at a time, from the middle
+      const int j = h ? n - 1 - i : i;
+      if (h ? j > tw : j < tw) sp_cp_async16(reinterpret_cast<char*>(cc) + (size_t)j * 128 + 16 * c, cs + (size_t)j * P * 8 + 16 * c);
+    }
+    sp_commit();
   }
-  dfl x = d;
-  sp[2 * (base + (size_t)(ny - 1) * P)] = x.h * sc;
-  // back substitution over rows j1, j1 - 1, ..., j1 - kDfCH + 1 (those >= 0)
-  auto load_b = [&](int j1, float2 (&dd)[kDfCH], float2 (&cc)[kDfCH]) {
+  for (int j = t; j < n; j += 32) {
+    ee[j] = f.a[j];
+    ee[n + j] = f.c[j];
+  }
+  __syncwarp();
+  const int rows = half ? n - 1 - tw : tw, j0 = half ? n - 1 : 0, dj = half ? -1 : 1;
+  const int s16 = 16 * dj;
+  float2 *pr = rr + j0 * 16 + q, *pi = iv + j0 * 16 + q;
+  const float2* po = ee + (half ? n : 0) + j0;
+  const bool pin = neumann && half == 0 && p0 + q == 0;
+  df2 d{f2(0.f), f2(0.f)};
+  for (int i = 0; i < most; i += kSpRows) {
+    if (i % per == 0) {
+      sp_wait_group(i / per);
+      __syncwarp();   // every lane's copies of the group
+    }
+    if (i + kSpRows <= rows) {
+      float2 r[kSpRows], v[kSpRows], o[kSpRows];
 #pragma unroll
-    for (int u = 0; u < kDfCH; ++u)
-      if (j1 - u >= 0) {
-        const size_t o = base + (size_t)(j1 - u) * P;
-        dd[u] = dp[2 * o];
-        cc[u] = cprF[o];
+      for (int u = 0; u < kSpRows; ++u) {
+        r[u] = pr[u * s16];
+        v[u] = pi[u * s16];
+        o[u] = po[u * dj];
       }
-  };
-  auto comp_b = [&](int j1, const float2 (&dd)[kDfCH], const float2 (&cc)[kDfCH], dfl x) {
+      if (pin && i == 0) r[0] = f2(0.f);
 #pragma unroll
-    for (int u = 0; u < kDfCH; ++u) {
-      const int j = j1 - u;
-      if (j >= 0) {
-        x = df_sub_mul(dfl{dd[u].x, dd[u].y}, dfl{cc[u].x, cc[u].y}, x);
-        sp[2 * (base + (size_t)j * P)] = x.h * sc;
+      for (int u = 0; u < kSpRows; ++u) {
+        d = df2_mul(df2_sub_mul(r[u], dfl{o[u].x, o[u].y}, d), dfl{v[u].x, v[u].y});
+        pr[u * s16] = d.h;
+        pi[u * s16] = d.l;
+      }
+    } else {
+      for (int u = 0; u < kSpRows && i + u < rows; ++u) {
+        const float2 r = pin && i + u == 0 ? f2(0.f) : pr[u * s16], v = pi[u * s16], o = po[u * dj];
+        d = df2_mul(df2_sub_mul(r, dfl{o.x, o.y}, d), dfl{v.x, v.y});
+        pr[u * s16] = d.h;
+        pi[u * s16] = d.l;
       }
     }
-    return x;
+    pr += kSpRows * s16;
+    pi += kSpRows * s16;
+    po += kSpRows * dj;
+  }
+  sp_wait<0>();
+  __syncwarp();
+  // the middle row, by the lower lanes; both halves go on from its solution
+  const df2 du{make_float2(__shfl_down_sync(0xffffffffu, d.h.x, 16), __shfl_down_sync(0xffffffffu, d.h.y, 16)),
+               make_float2(__shfl_down_sync(0xffffffffu, d.l.x, 16), __shfl_down_sync(0xffffffffu, d.l.y, 16))};
+  const bool store = (p0 + q) % g.mp < (size_t)g.mh && !(skip_mean && p0 + q == 0);
+  float2* out = reinterpret_cast<float2*>(spec + p0) + q;
+  df2 x;
+  {
+    const float2 r = rr[tw * 16 + q], v = iv[tw * 16 + q], a = ee[tw], c = ee[n + tw];
+    x = df2_mul(df2_sub_mul(df2_sub_mul(r, dfl{a.x, a.y}, d), dfl{c.x, c.y}, du), dfl{v.x, v.y});
+    if (store && half == 0) out[(size_t)tw * P] = __fmul2_rn(x.h, f2(sc));
+    x.h = make_float2(__shfl_sync(0xffffffffu, x.h.x, q), __shfl_sync(0xffffffffu, x.h.y, q));
+    x.l = make_float2(__shfl_sync(0xffffffffu, x.l.x, q), __shfl_sync(0xffffffffu, x.l.y, q));
+  }
+  // back substitution, away from the middle
+  const int jl = half ? tw + 1 : tw - 1;   // the last row eliminated
+  const float2 *bh = rr + jl * 16 + q, *bl = iv + jl * 16 + q, *bc = cc + jl * 16 + q;
+  float2* po2 = out + (ptrdiff_t)jl * (ptrdiff_t)P;
+  const ptrdiff_t step = -(ptrdiff_t)dj * (ptrdiff_t)P;
+  int i = rows;
+  for (; i >= kSpRows; i -= kSpRows) {
+    float2 h[kSpRows], l[kSpRows], c[kSpRows];
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u) {
+      h[u] = bh[-u * s16];
+      l[u] = bl[-u * s16];
+      c[u] = bc[-u * s16];
+    }
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u) {
+      x = df2_sub_mul(df2{h[u], l[u]}, dfl{c[u].x, c[u].y}, x);
+      if (store) *po2 = __fmul2_rn(x.h, f2(sc));
+      po2 += step;
+    }
+    bh -= kSpRows * s16;
+    bl -= kSpRows * s16;
+    bc -= kSpRows * s16;
+  }
+  for (; i > 0; --i) {
+    x = df2_sub_mul(df2{*bh, *bl}, dfl{bc->x, bc->y}, x);
+    if (store) *po2 = __fmul2_rn(x.h, f2(sc));
+    po2 += step;
+    bh -= s16;
+    bl -= s16;
+    bc -= s16;
+  }
+}
+
+// The same, streamed: 32 points per block, warp 0 from the bottom wall and warp 1
+// from the top wall; rows come in double-buffered batches and the forward values
+// go through dscr.  For columns too long to keep enough blocks on an SM.
+__global__ void __launch_bounds__(64)
+    k_spec_df_stream(cplx<float>* __restrict__ spec, float4* __restrict__ dscr, SpecDF f, Geo g, float sc,
+                     bool neumann, bool skip_mean) {
+  __shared__ df2 xch[2][32];
+  const int n = g.nyc, tw = n / 2, half = threadIdx.x >> 5, q = threadIdx.x & 31;
+  const size_t P = (size_t)g.nz * g.mp, p = (size_t)blockIdx.x * 32 + q;
+  const int rows = half ? n - 1 - tw : tw;
+  const ptrdiff_t sP = half ? -(ptrdiff_t)P : (ptrdiff_t)P, j0 = half ? n - 1 : 0;
+  const int dj = half ? -1 : 1;
+  const float2* pr = reinterpret_cast<const float2*>(spec) + p + j0 * (ptrdiff_t)P;
+  const float2* pi = f.inv + p + j0 * (ptrdiff_t)P;
+  const float2* po = (half ? f.c : f.a) + j0;
+  float4* pd = dscr + p + j0 * (ptrdiff_t)P;
+  const bool pin = neumann && half == 0 && p == 0;
+  df2 d{f2(0.f), f2(0.f)};
+  auto load_f = [&](int i, float2 (&r)[kSpRows], float2 (&v)[kSpRows]) {   // the next batch, of rows from i
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i + u < rows) {
+        r[u] = pr[u * sP];
+        v[u] = pi[u * sP];
+      }
+    pr += kSpRows * sP;
+    pi += kSpRows * sP;
+  };
+  auto comp_f = [&](int i, const float2 (&r)[kSpRows], const float2 (&v)[kSpRows]) {
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i + u < rows) {
+        const float2 o = __ldg(po + u * dj);
+        d = df2_mul(df2_sub_mul(pin && i + u == 0 ? f2(0.f) : r[u], dfl{o.x, o.y}, d), dfl{v[u].x, v[u].y});
+        pd[u * sP] = make_float4(d.h.x, d.h.y, d.l.x, d.l.y);
+      }
+    po += kSpRows * dj;
+    pd += kSpRows * sP;
   };
   {
-    float2 dA[kDfCH], dB[kDfCH], cA[kDfCH], cB[kDfCH];
-    load_b(ny - 2, dA, cA);
-    for (int j1 = ny - 2; j1 >= 0; j1 -= 2 * kDfCH) {
-      if (j1 - kDfCH >= 0) load_b(j1 - kDfCH, dB, cB);
-      x = comp_b(j1, dA, cA, x);
-      if (j1 - kDfCH >= 0) {
-        if (j1 - 2 * kDfCH >= 0) load_b(j1 - 2 * kDfCH, dA, cA);
-        x = comp_b(j1 - kDfCH, dB, cB, x);
+    float2 rA[kSpRows], rB[kSpRows], vA[kSpRows], vB[kSpRows];
+    load_f(0, rA, vA);
+    for (int i = 0; i < rows; i += 2 * kSpRows) {
+      if (i + kSpRows < rows) load_f(i + kSpRows, rB, vB);
+      comp_f(i, rA, vA);
+      if (i + kSpRows < rows) {
+        if (i + 2 * kSpRows < rows) load_f(i + 2 * kSpRows, rA, vA);
+        comp_f(i + kSpRows, rB, vB);
+      }
+    }
+  }
+  if (half) xch[0][q] = d;
+  __syncthreads();
+  const bool store = p % g.mp < (size_t)g.mh && !(skip_mean && p == 0);
+  float2* out = reinterpret_cast<float2*>(spec) + p;
+  if (!half) {
+    const float2 r = out[(size_t)tw * P], v = f.inv[p + (size_t)tw * P], a = f.a[tw], c = f.c[tw];
+    const df2 x = df2_mul(df2_sub_mul(df2_sub_mul(r, dfl{a.x, a.y}, d), dfl{c.x, c.y}, xch[0][q]), dfl{v.x, v.y});
+    if (store) out[(size_t)tw * P] = __fmul2_rn(x.h, f2(sc));
+    xch[1][q] = x;
+  }
+  __syncthreads();
+  df2 x = xch[1][q];
+  const ptrdiff_t jl = half ? tw + 1 : tw - 1;
+  const float4* bd = dscr + p + jl * (ptrdiff_t)P;
+  const float2* bc = f.cpr + p + jl * (ptrdiff_t)P;
+  out += jl * (ptrdiff_t)P;
+  auto load_b = [&](int i, float4 (&dd)[kSpRows], float2 (&c)[kSpRows]) {   // i rows are left
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i - u > 0) {
+        dd[u] = bd[-u * sP];
+        c[u] = bc[-u * sP];
+      }
+    bd -= kSpRows * sP;
+    bc -= kSpRows * sP;
+  };
+  auto comp_b = [&](int i, const float4 (&dd)[kSpRows], const float2 (&c)[kSpRows]) {
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i - u > 0) {
+        x = df2_sub_mul(df2{make_float2(dd[u].x, dd[u].y), make_float2(dd[u].z, dd[u].w)}, dfl{c[u].x, c[u].y}, x);
+        if (store) out[-u * sP] = __fmul2_rn(x.h, f2(sc));
+      }
+    out -= kSpRows * sP;
+  };
+  {
+    float4 dA[kSpRows], dB[kSpRows];
+    float2 cA[kSpRows], cB[kSpRows];
+    load_b(rows, dA, cA);
+    for (int i = rows; i > 0; i -= 2 * kSpRows) {
+      if (i > kSpRows) load_b(i - kSpRows, dB, cB);
+      comp_b(i, dA, cA);
+      if (i > kSpRows) {
+        if (i > 2 * kSpRows) load_b(i - 2 * kSpRows, dA, cA);
+        comp_b(i - kSpRows, dB, cB);
       }
     }
   }
 }
 
-// The FP64 (0,0) mode of the mixed potential as one block.  All threads stage
-// the column in shared memory; both Thomas sweeps are first-order linear
-// recurrences x_j = A_j + B_j x_(j-1) (forward: A = src_j / pivot_j,
+// FP64, streamed: 16 points per block, real and imaginary parts in adjacent lanes,
+// warp 0 from the bottom wall and warp 1 from the top wall, the forward values
+// through dscr.  (Columns in shared memory gained nothing: 12.4 against 10.5 us
+// at 32x33x32, 28.8 against 28.7 us at 128x97x128, where the FP64 pipe bounds it.)
+__global__ void __launch_bounds__(64)
+    k_spec_f64(double* __restrict__ spec, double* __restrict__ dscr, const double* __restrict__ cprF,
+               const double* __restrict__ invF, const double* __restrict__ aF, const double* __restrict__ cF, Geo g,
+               double sc, bool neumann, bool skip_mean) {
+  __shared__ double xch[2][32];
+  const int n = g.nyc, tw = n / 2, half = threadIdx.x >> 5, t = threadIdx.x & 31, q = t >> 1;
+  const size_t P = (size_t)g.nz * g.mp, p = (size_t)blockIdx.x * 16 + q;
+  const int rows = half ? n - 1 - tw : tw, dj = half ? -1 : 1;
+  const ptrdiff_t sP = half ? -(ptrdiff_t)P : (ptrdiff_t)P, j0 = half ? n - 1 : 0;
+  const size_t p2 = (size_t)blockIdx.x * 32 + t;   // this lane's value of plane j at 2 j P + p2
+  const double *pr = spec + p2 + 2 * j0 * (ptrdiff_t)P, *pi = invF + p + j0 * (ptrdiff_t)P;
+  const double* po = (half ? cF : aF) + j0;
+  double* pd = dscr + p2 + 2 * j0 * (ptrdiff_t)P;
+  const bool pin = neumann && half == 0 && p == 0;
+  double d = 0.0;
+  auto load_f = [&](int i, double (&r)[kSpRows], double (&v)[kSpRows]) {   // the next batch, of rows from i
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i + u < rows) {
+        r[u] = pr[2 * u * sP];
+        v[u] = pi[u * sP];
+      }
+    pr += 2 * kSpRows * sP;
+    pi += kSpRows * sP;
+  };
+  auto comp_f = [&](int i, const double (&r)[kSpRows], const double (&v)[kSpRows]) {
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i + u < rows) {
+        d = ((pin && i + u == 0 ? 0.0 : r[u]) - __ldg(po + u * dj) * d) * v[u];
+        pd[2 * u * sP] = d;
+      }
+    po += kSpRows * dj;
+    pd += 2 * kSpRows * sP;
+  };
+  {
+    double rA[kSpRows], rB[kSpRows], vA[kSpRows], vB[kSpRows];
+    load_f(0, rA, vA);
+    for (int i = 0; i < rows; i += 2 * kSpRows) {
+      if (i + kSpRows < rows) load_f(i + kSpRows, rB, vB);
+      comp_f(i, rA, vA);
+      if (i + kSpRows < rows) {
+        if (i + 2 * kSpRows < rows) load_f(i + 2 * kSpRows, rA, vA);
+        comp_f(i + kSpRows, rB, vB);
+      }
+    }
+  }
+  if (half) xch[0][t] = d;
+  __syncthreads();
+  const bool store = p % g.mp < (size_t)g.mh && !(skip_mean && p == 0);
+  double* out = spec + p2;
+  if (!half) {
+    const double x = ((out[2 * (size_t)tw * P] - aF[tw] * d) - cF[tw] * xch[0][t]) * invF[p + (size_t)tw * P];
+    if (store) out[2 * (size_t)tw * P] = x * sc;
+    xch[1][t] = x;
+  }
+  __syncthreads();
+  double x = xch[1][t];
+  const ptrdiff_t jl = half ? tw + 1 : tw - 1;
+  const double *bd = dscr + p2 + 2 * jl * (ptrdiff_t)P, *bc = cprF + p + jl * (ptrdiff_t)P;
+  out += 2 * jl * (ptrdiff_t)P;
+  auto load_b = [&](int i, double (&dd)[kSpRows], double (&c)[kSpRows]) {   // i rows are left
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i - u > 0) {
+        dd[u] = bd[-2 * u * sP];
+        c[u] = bc[-u * sP];
+      }
+    bd -= 2 * kSpRows * sP;
+    bc -= kSpRows * sP;
+  };
+  auto comp_b = [&](int i, const double (&dd)[kSpRows], const double (&c)[kSpRows]) {
+#pragma unroll
+    for (int u = 0; u < kSpRows; ++u)
+      if (i - u > 0) {
+        x = dd[u] - c[u] * x;
+        if (store) out[-2 * u * sP] = x * sc;
+      }
+    out -= 2 * kSpRows * sP;
+  };
+  {
+    double dA[kSpRows], dB[kSpRows], cA[kSpRows], cB[kSpRows];
+    load_b(rows, dA, cA);
+    for (int i = rows; i > 0; i -= 2 * kSpRows) {
+      if (i > kSpRows) load_b(i - kSpRows, dB, cB);
+      comp_b(i, dA, cA);
+      if (i > kSpRows) {
+        if (i > 2 * kSpRows) load_b(i - 2 * kSpRows, dA, cA);
+        comp_b(i - kSpRows, dB, cB);
+      }
+    }
+  }
+}
+
+// The FP64 (0,0) mode of the mixed potential as one block: the FP32 transform's
+// mean of the fluctuating charge, scaled, plus the FP64 reference source; the
+// solution goes to mean_out (plus mean_shift) and the transform slots are zeroed.
+// All threads stage the column in shared memory; both Thomas sweeps are first-
+// order linear recurrences x_j = A_j + B_j x_(j-1) (forward: A = src_j / pivot_j,
 // B = -a_j / pivot_j; back substitution, run from the top: A = d_j, B = -c'_j),
 // so the first warp solves each as a scan of affine maps: every lane composes
 // the maps of its chunk of rows, a Kogge-Stone scan over the 32 lanes composes
@@ -1024,7 +1162,7 @@ __global__ void k_spec_thomas_df(cplx<float>* __restrict__ spec, float2* __restr
 // The dependent FP64 chain shrinks from two steps per row to ~2 n / 32 + 10
 // steps.  |B| < 1 on the diagonally dominant y-operator, so the composed
 // products only shrink.  Then all threads write the result and zero the
-// transform slots.
+// transform slots.  cpr, inv: the one-sided factors of this mode, per plane.
 constexpr int kMeanSmemRows = 640;   // 5 doubles per row: 25 KB of static shared memory
 
 // x_j = A_j + B_j x_(j-1) for j = 0 .. n-1 with x_(-1) = 0, by the first warp;
@@ -1056,28 +1194,64 @@ __device__ __forceinline__ void affine_scan_warp(int n, FA A, FB B, FX x) {
   }
 }
 
-__global__ void __launch_bounds__(256) k_spec_mean(cplx<float>* __restrict__ spec, const double* __restrict__ cpr,
+template <typename T>
+__global__ void __launch_bounds__(256) k_spec_mean(cplx<T>* __restrict__ spec, const double* __restrict__ cpr,
                                                    const double* __restrict__ inv, YRows rows, Geo g, double scale,
                                                    const double* __restrict__ mean_rhs,
                                                    const double* __restrict__ mean_shift,
                                                    double* __restrict__ mean_out) {
   const size_t P = (size_t)g.nz * g.mp;
   const int ny = g.nyc;
-  float* sp = reinterpret_cast<float*>(spec);   // (0,0) mode, real part at sp[2 j P], imaginary at sp[2 j P + 1]
-  if (ny > kMeanSmemRows) {
-    if (threadIdx.x < 2)
-      spec_mean_mode(sp + threadIdx.x, cpr, inv, rows, 0, P, ny, (int)threadIdx.x, scale, mean_rhs, mean_shift,
-                     mean_out);
+  T* sp = reinterpret_cast<T*>(spec);   // (0,0) mode, real part at sp[2 j P], imaginary at sp[2 j P + 1]
+  if (ny > kMeanSmemRows) {   // one thread walks the column, loads eight rows at a time
+    if (threadIdx.x == 0) {
+      constexpr int CH = 8;
+      double d = 0.0;
+      for (int j0 = 0; j0 < ny; j0 += CH) {
+        double r[CH], iv[CH], mr[CH];
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (j0 + u < ny) {
+            r[u] = (double)sp[2 * (size_t)(j0 + u) * P];
+            iv[u] = inv[j0 + u];
+            mr[u] = mean_rhs[j0 + u];
+          }
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (j0 + u < ny) {
+            d = (r[u] * scale + mr[u] - rows.a[j0 + u] * d) * iv[u];
+            mean_out[j0 + u] = d;
+          }
+      }
+      double x = 0.0;
+      for (int j1 = ny - 1; j1 >= 0; j1 -= CH) {
+        double dd[CH], c[CH], sh[CH];
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (j1 - u >= 0) {
+            dd[u] = mean_out[j1 - u];
+            c[u] = j1 - u < ny - 1 ? cpr[j1 - u] : 0.0;
+            sh[u] = mean_shift[j1 - u];
+          }
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+          if (j1 - u >= 0) {
+            x = dd[u] - c[u] * x;
+            mean_out[j1 - u] = x + sh[u];
+          }
+      }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < ny; j += blockDim.x) sp[2 * (size_t)j * P] = sp[2 * (size_t)j * P + 1] = T(0);
     return;
   }
   __shared__ double e[kMeanSmemRows], fa[kMeanSmemRows], cp[kMeanSmemRows], ms[kMeanSmemRows],
       out[kMeanSmemRows];
   for (int j = threadIdx.x; j < ny; j += blockDim.x) {
-    const size_t o = (size_t)j * P;
-    const double iv = inv[o];
-    e[j] = ((double)sp[2 * o] * scale + mean_rhs[j]) * iv;
+    const double iv = inv[j];
+    e[j] = ((double)sp[2 * (size_t)j * P] * scale + mean_rhs[j]) * iv;
     fa[j] = rows.a[j] * iv;
-    cp[j] = cpr[o];
+    cp[j] = cpr[j];
     ms[j] = mean_shift[j];
   }
   __syncthreads();
@@ -1093,140 +1267,64 @@ __global__ void __launch_bounds__(256) k_spec_mean(cplx<float>* __restrict__ spe
   }
   __syncthreads();
   for (int j = threadIdx.x; j < ny; j += blockDim.x) {
-    const size_t o = (size_t)j * P;
     mean_out[j] = out[j] + ms[j];
-    sp[2 * o] = 0.f;
-    sp[2 * o + 1] = 0.f;
+    sp[2 * (size_t)j * P] = T(0);
+    sp[2 * (size_t)j * P + 1] = T(0);
   }
 }
 
-// The same df elimination with the forward values in shared memory.  One warp
-// owns 8 consecutive spectral points m of two z-wavenumbers n (16 points, real
-// and imaginary part in adjacent lanes); the right-hand sides and 1/pivot of
-// the forward sweep, then c' of the back substitution, stream through a
-// two-chunk cp.async ring (16 planes per chunk, the back-substitution chunks
-// following the forward ones without a gap), and the df values d_j stay in
-// shared memory, so the sweep scratch never reaches HBM.  Same operations in
-// the same order as k_spec_thomas_df.
-constexpr int kSpChunk = 16;
-
-__host__ __device__ inline size_t spec_tile_bytes(int n) {
-  // d [n][32] float2, r ring [2][kSpChunk][32] float, factor ring [2][kSpChunk][16] float2, a [n] float2
-  return (size_t)n * 32 * 8 + 2 * kSpChunk * 32 * 4 + 2 * kSpChunk * 16 * 8 + (size_t)n * 8;
+// Columns in shared memory (launch code 16) or streamed (32); 0 and the other
+// codes: in shared memory where all blocks are resident at once.  There the solve
+// is one column's latency, on one wave: 13.2 against 15.2 us at 64x65x64 (19.6
+// streamed one-sided), 17.4 against 27.6 at 128x97x128, 29.0 against 58.4 at
+// 64x257x64.  Over more waves the few warps that the columns leave room for lose to
+// the bandwidth of many streams, and so they do beside other cases' kernels
+// (ensembles, whose waves add up, take the streamed form): 100.8 against 74.1 us at 256x193x256 (5.5 TB/s;
+// 105.3 one-sided, scalar), 136 against 91 at 128x385x128.
+double spec_smem_waves(const Geo& g) {
+  constexpr size_t kMost = 227 * 1024;
+  const size_t need = spec_smem_df(g.nyc);
+  int dev = 0, sms = 0;
+  if (need > kMost || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1e30;
+  const size_t per_sm = kMost / (need + 1024);   // 1 KB per block is the system's
+  return (double)g.nz * g.mp / 16 / ((double)sms * (per_sm < 1 ? 1 : per_sm < 32 ? per_sm : 32));
 }
 
-__device__ __forceinline__ void sp_cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
+template <typename T>
+static cudaError_t launch_spec_mean(cplx<T>* spec, const YRows& rows, const Geo& g, double scale, cudaStream_t s,
+                                    const SpecMean* m) {
+  if (!m) return cudaSuccess;
+  k_spec_mean<T><<<1, 256, 0, s>>>(spec, m->cpr, m->inv, rows, g, scale, m->rhs, m->shift, m->out);
+  return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(32) k_spec_thomas_tile(cplx<float>* __restrict__ spec, SpecDF f, Geo g, float sc,
-                                                         bool neumann, bool skip_mean) {
-  extern __shared__ __align__(16) unsigned char sp_smem[];
-  const int n = g.nyc;
-  float2* dd = reinterpret_cast<float2*>(sp_smem);              // [n][32]
-  float* rr = reinterpret_cast<float*>(dd + (size_t)n * 32);    // [2][kSpChunk][32]
-  float2* ff = reinterpret_cast<float2*>(rr + 2 * kSpChunk * 32);   // [2][kSpChunk][16]
-  float2* aa = ff + 2 * kSpChunk * 16;                          // [n]
-  const int t = threadIdx.x, part = t & 1, q = t >> 1, rs = q >> 3, mq = q & 7;
-  const int m0 = blockIdx.x * 8, n0 = blockIdx.y * 2;
-  const int m = m0 + mq, nn = n0 + rs;
-  const size_t P = (size_t)g.nz * g.mp;   // complex values per plane
-  const float* specf = reinterpret_cast<const float*>(spec);
-  const int K = (n + kSpChunk - 1) / kSpChunk;
-  // step s < K: forward chunk s (r and 1/pivot of planes [16 s, 16 s + 16));
-  // step s >= K: back-substitution chunk b = s - K (c' of planes [hi - 16, hi), hi = n - 16 b)
-  auto issue = [&](int st) {
-    if (st < 2 * K) {
-      const bool fwd = st < K;
-      const int b = fwd ? st : st - K;
-      const int hi = fwd ? min(n, (b + 1) * kSpChunk) : n - b * kSpChunk;
-      const int lo = fwd ? b * kSpChunk : max(0, hi - kSpChunk);
-      float* rb = rr + (st & 1) * kSpChunk * 32;
-      float2* fb = ff + (st & 1) * kSpChunk * 16;
-      const float2* fac = fwd ? f.inv : f.cpr;
-      for (int e = t; e < (hi - lo) * 8; e += 32) {
-        const int jj = e >> 3, sr = (e >> 2) & 1, c = e & 3;
-        const int j = fwd ? lo + jj : hi - 1 - jj;
-        const size_t o = (size_t)j * P + (size_t)(n0 + sr) * g.mp + m0;   // complex index of the row segment
-        if (fwd) sp_cp_async16(rb + jj * 32 + sr * 16 + c * 4, specf + 2 * o + c * 4);
-        sp_cp_async16(fb + jj * 16 + sr * 8 + c * 2, fac + o + c * 2);
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  issue(0);
-  issue(1);
-  for (int j = t; j < n; j += 32) aa[j] = f.a[j];
-  const bool pin = neumann && m == 0 && nn == 0;
-  dfl d{0.f, 0.f};
-  for (int st = 0; st < K; ++st) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp();
-    const float* rb = rr + (st & 1) * kSpChunk * 32;
-    const float2* fb = ff + (st & 1) * kSpChunk * 16;
-    const int lo = st * kSpChunk, hi = min(n, lo + kSpChunk);
-    for (int j = lo; j < hi; ++j) {
-      const int jj = j - lo;
-      const float r = (pin && j == 0) ? 0.f : rb[jj * 32 + t];
-      const float2 a = aa[j], iv = fb[jj * 16 + q];
-      d = df_mul(df_sub_mul(r, dfl{a.x, a.y}, d), dfl{iv.x, iv.y});
-      dd[(size_t)j * 32 + t] = make_float2(d.h, d.l);
-    }
-    __syncwarp();
-    issue(st + 2);
-  }
-  const bool store = m < g.mh && !(skip_mean && m == 0 && nn == 0);
-  float* out = reinterpret_cast<float*>(spec) + 2 * ((size_t)nn * g.mp + m) + part;   // plane j at out[2 j P]
-  dfl x = d;
-  for (int b = 0; b < K; ++b) {
-    const int st = K + b;
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp();
-    const float2* fb = ff + (st & 1) * kSpChunk * 16;
-    const int hi = n - b * kSpChunk, lo = max(0, hi - kSpChunk);
-    for (int j = hi - 1; j >= lo; --j) {
-      if (j < n - 1) {
-        const float2 dj = dd[(size_t)j * 32 + t], cp = fb[(hi - 1 - j) * 16 + q];
-        x = df_sub_mul(dfl{dj.x, dj.y}, dfl{cp.x, cp.y}, x);
-      }
-      if (store) out[2 * (size_t)j * P] = x.h * sc;
-    }
-    __syncwarp();
-    issue(st + 2);
-  }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-}
-
-cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f, const double* cpr,
-                                  const double* inv, const YRows& rows, const Geo& g, double scale, bool neumann,
-                                  cudaStream_t s, const double* mean_rhs, const double* mean_shift,
-                                  double* mean_out) {
-  if (mean_rhs != nullptr) {
-    k_spec_mean<<<1, 256, 0, s>>>(spec, cpr, inv, rows, g, scale, mean_rhs, mean_shift, mean_out);
-    const cudaError_t e = cudaGetLastError();
+cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f, const YRows& rows, const Geo& g,
+                                  double scale, bool neumann, cudaStream_t s, const SpecMean* mean) {
+  cudaError_t e = launch_spec_mean(spec, rows, g, scale, s, mean);
+  if (e != cudaSuccess) return e;
+  const unsigned n16 = (unsigned)((size_t)g.nz * g.mp / 16);   // nz a multiple of 4, mp of 8
+  const size_t need = spec_smem_df(g.nyc);
+  if (g.lc_spec == 16 ? need <= 227 * 1024 : g.lc_spec != 32 && spec_smem_waves(g) <= 1.0) {
+    if (need > 48 * 1024) e = cudaFuncSetAttribute(k_spec_df_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (e != cudaSuccess) return e;
+    k_spec_df_smem<<<n16, 32, need, s>>>(spec, f, g, (float)scale, neumann, mean != nullptr);
+  } else {
+    k_spec_df_stream<<<n16 / 2, 64, 0, s>>>(spec, reinterpret_cast<float4*>(dscr), f, g, (float)scale, neumann,
+                                            mean != nullptr);
   }
-  // shared-memory tiles (lc_spec 16) when 8-point row segments tile the padded
-  // pitch, the z-wavenumbers pair up and a column block fits.  Measured on the
-  // 256x193x256 workload: 0.18 ms against 0.10 ms for one thread per point --
-  // the ~48 KB of df forward values per warp leaves three warps per SM to hide
-  // the double-float dependency chain -- so it is only an autotuner candidate.
-  const size_t tbytes = spec_tile_bytes(g.nyc);
-  if (g.lc_spec == 16 && g.mp % 8 == 0 && g.nz % 2 == 0 && tbytes <= 227 * 1024) {
-    if (tbytes > 48 * 1024) {
-      const cudaError_t e =
-          cudaFuncSetAttribute(k_spec_thomas_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tbytes);
-      if (e != cudaSuccess) return e;
-    }
-    const dim3 grd((unsigned)((g.mh + 7) / 8), (unsigned)(g.nz / 2));
-    k_spec_thomas_tile<<<grd, 32, tbytes, s>>>(spec, f, g, (float)scale, neumann, mean_rhs != nullptr);
-    return cudaGetLastError();
-  }
-  const int T_ = g.lc_spec ? g.lc_spec : 64;
-  dim3 grd((2 * g.mh + T_ - 1) / T_, g.nz, 1);
-  k_spec_thomas_df<<<grd, T_, 0, s>>>(spec, reinterpret_cast<float2*>(dscr), f.cpr, f.inv, f.a, cpr, inv, rows, g,
-                                      scale, (float)scale, neumann, mean_rhs, mean_shift, mean_out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_spec_thomas(cplx<double>* spec, cplx<double>* dscr, const double* cpr, const double* inv,
+                               const YRows& rows, const Geo& g, double scale, bool neumann, cudaStream_t s,
+                               const SpecMean* mean) {
+  const cudaError_t e = launch_spec_mean(spec, rows, g, scale, s, mean);
+  if (e != cudaSuccess) return e;
+  k_spec_f64<<<(unsigned)((size_t)g.nz * g.mp / 16), 64, 0, s>>>(
+      reinterpret_cast<double*>(spec), reinterpret_cast<double*>(dscr), cpr, inv, rows.a, rows.c, g, scale, neumann,
+      mean != nullptr);
   return cudaGetLastError();
 }
 
@@ -1629,13 +1727,6 @@ template cudaError_t launch_fft_x_fwd<double, float>(PoissonSrc, const float*, c
 
 template cudaError_t launch_fft_z<double>(cplx<double>*, const cplx<double>*, const Geo&, bool, cudaStream_t);
 template cudaError_t launch_fft_z<float>(cplx<float>*, const cplx<float>*, const Geo&, bool, cudaStream_t);
-
-template cudaError_t launch_spec_thomas<double>(cplx<double>*, cplx<double>*, const double*, const double*,
-                                                const YRows&, const Geo&, double, bool, cudaStream_t,
-                                                const double*, const double*, double*);
-template cudaError_t launch_spec_thomas<float>(cplx<float>*, cplx<double>*, const double*, const double*,
-                                               const YRows&, const Geo&, double, bool, cudaStream_t,
-                                               const double*, const double*, double*);
 
 template cudaError_t launch_fft_x_inv<double, double>(PoissonDst, const cplx<double>*, const Geo&, const Metrics&,
                                                       const cplx<double>*, const cplx<double>*, double, double*,

@@ -96,7 +96,8 @@ struct pnp_ctx {
   double *spc_cprN, *spc_invN, *spc_cprD, *spc_invD;
   // mixed path: their double-float copies and the y-operator sub-diagonals as df
   float2 *spf_cprN = nullptr, *spf_invN = nullptr, *spf_cprD = nullptr, *spf_invD = nullptr;
-  float2 *spf_aN = nullptr, *spf_aD = nullptr;
+  float2 *spf_aN = nullptr, *spf_aD = nullptr;   // sub-, then super-diagonal ([2][ny])
+  double* mean_fac = nullptr;                    // one-sided factors c', 1/pivot of the (0,0) Dirichlet mode ([2][ny])
   // mixed path: low parts of the ion fluctuations (c = c_ref + S + L, S the shadow)
   float *cpL = nullptr, *cmL = nullptr;
   float2 *dCp_f2 = nullptr, *dCm_f2 = nullptr;   // [3][ny] reference increments as df pairs
@@ -227,7 +228,8 @@ size_t carve(pnp_ctx* c, char* base, int nx, int ny, int nz, int precision) {
   const bool mixed = precision == PNP_MIXED;
   float2 *sfcN = b.take<float2>(mixed ? nspec : 0), *sfiN = b.take<float2>(mixed ? nspec : 0);
   float2 *sfcD = b.take<float2>(mixed ? nspec : 0), *sfiD = b.take<float2>(mixed ? nspec : 0);
-  float2 *sfaN = b.take<float2>(mixed ? ny : 0), *sfaD = b.take<float2>(mixed ? ny : 0);
+  float2 *sfaN = b.take<float2>(mixed ? 2 * ny : 0), *sfaD = b.take<float2>(mixed ? 2 * ny : 0);
+  double* mfac = b.take<double>(2 * (size_t)ny);
   float *cpL = b.take<float>(mixed ? nc : 0), *cmL = b.take<float>(mixed ? nc : 0);
   float2 *dCp2 = b.take<float2>(3 * (size_t)ny), *dCm2 = b.take<float2>(3 * (size_t)ny);
   double *wB = b.take<double>((size_t)nz * nx), *wT = b.take<double>((size_t)nz * nx);
@@ -246,6 +248,7 @@ size_t carve(pnp_ctx* c, char* base, int nx, int ny, int nz, int precision) {
     c->dCp_f2 = dCp2; c->dCm_f2 = dCm2;
     c->spf_cprN = sfcN; c->spf_invN = sfiN; c->spf_cprD = sfcD; c->spf_invD = sfiD;
     c->spf_aN = sfaN; c->spf_aD = sfaD;
+    c->mean_fac = mfac;
     c->cpL = cpL; c->cmL = cmL;
     c->dscr = dscr;
     c->spec2 = spec2;
@@ -353,6 +356,13 @@ int upload_metrics(pnp_ctx* c) {
       else if (bc == 1) b[j] -= hi;
     }
   }
+  std::vector<double> mfac(2 * (size_t)ny, 0.0);   // Thomas factors of the constant mode between Dirichlet walls
+  for (int j = 0; j < nyc; ++j) {
+    const double *a = rD.data(), *b = a + ny, *cc = b + ny;
+    const double iv = 1.0 / (b[j] - (j ? a[j] * mfac[j - 1] : 0.0));
+    mfac[j] = cc[j] * iv;
+    mfac[ny + j] = iv;
+  }
   const int nx = c->g.nx, nz = c->g.nz, mh = c->g.mh, mp = c->g.mp;
   std::vector<double> kx2(mp, 0.0), kz2(nz, 0.0);
   for (int m = 0; m < mh; ++m) kx2[m] = (2.0 - 2.0 * std::cos(2.0 * M_PI * m / nx)) / (c->g.dx * c->g.dx);
@@ -384,6 +394,7 @@ int upload_metrics(pnp_ctx* c) {
   CK(up(c->wu_d, wu.data(), B));
   CK(up(c->rowsN_d, rN.data(), 3 * B));
   CK(up(c->rowsD_d, rD.data(), 3 * B));
+  CK(up(c->mean_fac, mfac.data(), 2 * B));
   CK(up(c->kx2_d, kx2.data(), sizeof(double) * mp));
   CK(up(c->kz2_d, kz2.data(), sizeof(double) * nz));
   CK(up(c->twx_d, twx.data(), sizeof(cplx<double>) * Lh));
@@ -418,7 +429,9 @@ int upload_metrics(pnp_ctx* c) {
       CK(launch_to_df(c->spc_cprD, c->spf_cprD, nspec, s));
       CK(launch_to_df(c->spc_invD, c->spf_invD, nspec, s));
       CK(launch_to_df(c->rowsN_d, c->spf_aN, (size_t)ny, s));
+      CK(launch_to_df(c->rowsN_d + 2 * (size_t)ny, c->spf_aN + ny, (size_t)ny, s));
       CK(launch_to_df(c->rowsD_d, c->spf_aD, (size_t)ny, s));
+      CK(launch_to_df(c->rowsD_d + 2 * (size_t)ny, c->spf_aD + ny, (size_t)ny, s));
     }
   }
   CK(cudaStreamSynchronize(s));   // host vectors above are temporaries
@@ -752,7 +765,13 @@ MixedRefs mixed_refs(const pnp_ctx* c) {
 }
 
 SpecDF spec_df(const pnp_ctx* c, bool neumann) {
-  return neumann ? SpecDF{c->spf_cprN, c->spf_invN, c->spf_aN} : SpecDF{c->spf_cprD, c->spf_invD, c->spf_aD};
+  const float2* a = neumann ? c->spf_aN : c->spf_aD;
+  return neumann ? SpecDF{c->spf_cprN, c->spf_invN, a, a + c->g.ny} : SpecDF{c->spf_cprD, c->spf_invD, a, a + c->g.ny};
+}
+
+// the (0,0) mode of a potential solve about the reference profiles
+SpecMean spec_mean(const pnp_ctx* c) {
+  return SpecMean{c->mean_fac, c->mean_fac + c->g.ny, c->meanrhs_d, c->meanshift_d, c->delta_d};
 }
 
 YRows yrows(const pnp_ctx* c, bool neumann) {
@@ -782,10 +801,9 @@ cudaError_t spectral_solve(pnp_ctx* c, cplx<T>* spec, const cplx<T>* twz, bool n
   mark(c, st, neumann ? PNP_SITE_P_FFTZ : PNP_SITE_E_FFTZ);
   const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
   if constexpr (sizeof(T) == sizeof(float))
-    e = launch_spec_thomas_df(spec, dscr, spec_df(c, neumann), neumann ? c->spc_cprN : c->spc_cprD,
-                              neumann ? c->spc_invN : c->spc_invD, yrows(c, neumann), c->g, scale, neumann, st);
+    e = launch_spec_thomas_df(spec, dscr, spec_df(c, neumann), yrows(c, neumann), c->g, scale, neumann, st);
   else
-    e = launch_spec_thomas<T>(spec, dscr, neumann ? c->spc_cprN : c->spc_cprD, neumann ? c->spc_invN : c->spc_invD,
+    e = launch_spec_thomas(spec, dscr, neumann ? c->spc_cprN : c->spc_cprD, neumann ? c->spc_invN : c->spc_invD,
                               yrows(c, neumann), c->g, scale, neumann, st);
   if (e != cudaSuccess) return e;
   mark(c, st, neumann ? PNP_SITE_P_THOMAS : PNP_SITE_E_THOMAS);
@@ -866,8 +884,8 @@ cudaError_t potential_mixed(pnp_ctx* c, cudaStream_t st, void* spec_buf, cplx<do
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_FFTZ);
   const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
-  e = launch_spec_thomas_df(spec, dscr, spec_df(c, false), c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale,
-                            false, st, c->meanrhs_d, c->meanshift_d, c->delta_d);
+  const SpecMean mean = spec_mean(c);
+  e = launch_spec_thomas_df(spec, dscr, spec_df(c, false), yrows(c, false), c->g, scale, false, st, &mean);
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_THOMAS);
   e = launch_fft_z<float>(spec, twz, c->g, true, st);
@@ -921,8 +939,8 @@ cudaError_t potential_mixed_fp64(pnp_ctx* c, cudaStream_t st, void* spec_buf, cp
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_FFTZ);
   const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
-  e = launch_spec_thomas<double>(spec, dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale, false, st,
-                                 c->meanrhs_d, c->meanshift_d, c->delta_d);
+  const SpecMean mean = spec_mean(c);
+  e = launch_spec_thomas(spec, dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale, false, st, &mean);
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_THOMAS);
   e = launch_fft_z<double>(spec, twz, c->g, true, st);
@@ -2055,17 +2073,17 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
     if (t < best[1]) { best[1] = t; pick[1] = T; }
   }
   c->g.lc_cn = pick[1];
-  // 3: spectral y-solve block size, 4: z-transform threads per column
+  // 3: spectral y-solve (columns in shared memory or streamed), 4: z-transform threads per column
   const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
-  for (int T : {16, 32, 64, 128}) {   // mixed: 16 = shared-memory tiles
+  for (int T : {16, 32}) {   // (FP64 has the streamed form only)
     c->g.lc_spec = T;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64)
-        launch_spec_thomas<double>((cplx<double>*)c->spec, c->dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g,
-                                   scale, false, c->stream);
+        launch_spec_thomas((cplx<double>*)c->spec, c->dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale,
+                           false, c->stream);
       else
-        launch_spec_thomas_df((cplx<float>*)c->spec, c->dscr, spec_df(c, false), c->spc_cprD, c->spc_invD,
-                              yrows(c, false), c->g, scale, false, c->stream);
+        launch_spec_thomas_df((cplx<float>*)c->spec, c->dscr, spec_df(c, false), yrows(c, false), c->g, scale, false,
+                              c->stream);
     }, reps);
     if (t < best[2]) { best[2] = t; pick[2] = T; }
   }
@@ -2119,7 +2137,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
       *f[i] = v;
     };
     float cur = step_ms();
-    const std::vector<int> cands[4] = {{32, 64, 128, 16}, {32, 64, 128, 256}, {16, 32, 64, 128}, {8, 16, 32, 64}};
+    const std::vector<int> cands[4] = {{32, 64, 128, 16}, {32, 64, 128, 256}, {16, 32}, {8, 16, 32, 64}};
     for (int i = 0; i < 4; ++i) {
       for (int v : cands[i]) {
         if (v == pick[i]) continue;
@@ -2242,17 +2260,23 @@ int pnp_ensemble_step(pnp_ensemble* e, int nsteps, const double* dt) {
     if (e->exec) cudaGraphExecDestroy(e->exec);
     e->exec = nullptr;
     cudaGraph_t graph = nullptr;
+    double waves = 0.0;   // the cases' spectral solves run side by side
+    for (int i = 0; i < n; ++i)
+      if (e->cases[i]->precision == PNP_MIXED) waves += spec_smem_waves(e->cases[i]->g);
     CK(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeRelaxed));
     cudaError_t err = cudaEventRecord(e->fork, e->stream);
     for (int i = 0; i < n && err == cudaSuccess; ++i) {
       pnp_ctx* c = e->cases[i];
       cudaStream_t own = c->stream;
+      const int own_spec = c->g.lc_spec;
+      if (waves > 1.0 && own_spec != 16) c->g.lc_spec = 32;
       c->stream = e->branch[i];   // the case's launches go to its capture branch
       err = cudaStreamWaitEvent(c->stream, e->fork, 0);
       if (err == cudaSuccess) err = one_step(c, dt[i]);
       if (err == cudaSuccess) err = cudaEventRecord(e->join[i], c->stream);
       if (err == cudaSuccess) err = cudaStreamWaitEvent(e->stream, e->join[i], 0);
       c->stream = own;
+      c->g.lc_spec = own_spec;
     }
     cudaError_t err2 = cudaStreamEndCapture(e->stream, &graph);
     if (err != cudaSuccess || err2 != cudaSuccess) {

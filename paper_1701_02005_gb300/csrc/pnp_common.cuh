@@ -33,7 +33,7 @@ struct Geo {
                          // mixed stencil: 128 TMA rows, 64 / 32 packed-pair cp.async tiles 64 / 32
                          // cells wide, 16 one-cell tiles
   int lc_cn;             // threads per block of the wall-normal CN sweeps (mixed: 32 = shared-memory line tiles)
-  int lc_spec;           // threads per block of the spectral y-solves (mixed: 16 = shared-memory tiles)
+  int lc_spec;           // spectral y-solves (mixed): 16 = columns in shared memory, 32 = streamed, else by size
   int lc_fftz_ty;        // threads per column of the z-transform (cap)
 };
 
@@ -171,18 +171,22 @@ cudaError_t launch_spec_factors(double* cpr, double* inv, const double* kx2, con
 // Double-float copies of the spectral elimination factors (mixed path).
 struct SpecDF {
   const float2 *cpr, *inv;   // per spectral point, same layout as the FP64 factors
-  const float2* a;           // sub-diagonal of the y-operator per plane
+  const float2 *a, *c;       // sub- and super-diagonal of the y-operator per plane
 };
-cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f, const double* cpr,
-                                  const double* inv, const YRows& rows, const Geo& g, double scale, bool neumann,
-                                  cudaStream_t s, const double* mean_rhs = nullptr,
-                                  const double* mean_shift = nullptr, double* mean_out = nullptr);
+// The FP64 (0,0) mode of the mixed potential: its one-sided elimination factors,
+// reference source, shift and solution, per plane.
+struct SpecMean {
+  const double *cpr, *inv, *rhs, *shift;
+  double* out;
+};
+cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f, const YRows& rows, const Geo& g,
+                                  double scale, bool neumann, cudaStream_t s, const SpecMean* mean = nullptr);
+// Waves of blocks of a mixed solve with its columns in shared memory.
+double spec_smem_waves(const Geo& g);
 cudaError_t launch_to_df(const double* x, float2* out, size_t n, cudaStream_t s);
-template <typename T>
-cudaError_t launch_spec_thomas(cplx<T>* spec, cplx<double>* dscr, const double* cpr, const double* inv,
+cudaError_t launch_spec_thomas(cplx<double>* spec, cplx<double>* dscr, const double* cpr, const double* inv,
                                const YRows& rows, const Geo& g, double scale, bool neumann, cudaStream_t s,
-                               const double* mean_rhs = nullptr, const double* mean_shift = nullptr,
-                               double* mean_out = nullptr);
+                               const SpecMean* mean = nullptr);
 
 // Potential / PotentialShadow: out = V yc_j (Potential) or plane_add[j]
 // (PotentialShadow) + the transform + cell_add[c] (optional, per cell).

@@ -89,6 +89,47 @@ __device__ __forceinline__ dfl df_prod(float a, float b) {
   return {p, __fmaf_rn(a, b, -p)};
 }
 
+// Two df values side by side (the real and imaginary part of a complex value) in
+// packed FP32: the same operations in the same order as above, so each lane
+// equals the scalar result bit for bit (a - b as fma(b, -1, a): one rounding).
+struct df2 {
+  float2 h, l;
+};
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.f), a); }
+__device__ __forceinline__ df2 df2_two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  const float2 bb = sub2(s, a);
+  return {s, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ df2 df2_mul(df2 a, dfl b) {
+  const float2 bh = f2(b.h), p = __fmul2_rn(a.h, bh);
+  float2 e = __ffma2_rn(a.h, bh, __fmul2_rn(p, f2(-1.f)));
+  e = __ffma2_rn(a.h, f2(b.l), e);
+  e = __ffma2_rn(a.l, bh, e);
+  const float2 s = __fadd2_rn(p, e);
+  return {s, sub2(e, sub2(s, p))};
+}
+// b * a with b the first factor of df_mul (the order of the cross terms)
+__device__ __forceinline__ df2 df2_mul(dfl b, df2 a) {
+  const float2 bh = f2(b.h), p = __fmul2_rn(bh, a.h);
+  float2 e = __ffma2_rn(bh, a.h, __fmul2_rn(p, f2(-1.f)));
+  e = __ffma2_rn(bh, a.l, e);
+  e = __ffma2_rn(f2(b.l), a.h, e);
+  const float2 s = __fadd2_rn(p, e);
+  return {s, sub2(e, sub2(s, p))};
+}
+__device__ __forceinline__ df2 df2_sub_mul(float2 r, dfl a, df2 b) {
+  const df2 p = df2_mul(a, b);
+  const df2 s = df2_two_sum(r, __fmul2_rn(p.h, f2(-1.f)));
+  return df2_two_sum(s.h, sub2(s.l, p.l));
+}
+__device__ __forceinline__ df2 df2_sub_mul(df2 x, dfl a, df2 b) {
+  const df2 p = df2_mul(a, b);
+  const df2 s = df2_two_sum(x.h, __fmul2_rn(p.h, f2(-1.f)));
+  return df2_two_sum(s.h, __fadd2_rn(s.l, sub2(x.l, p.l)));
+}
+
 // Host-side split of a double into a df pair (hi = nearest float).
 inline dfl df_split_host(double x) {
   const float h = (float)x;
