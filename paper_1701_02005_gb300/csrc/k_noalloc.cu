@@ -176,7 +176,7 @@ extern "C" int pnp_poisson_noalloc(int nx, int ny, int nz, double Lx, double Lz,
                                        g, m, spec, tx, tp, s) != cudaSuccess)
     return PNP_ERR_CUDA;
   if (launch_fft_z<double>(spec, tz, g, false, s) != cudaSuccess) return PNP_ERR_CUDA;
-  const double scale = 1.0 / ((double)nx * (double)nz);
+  const double scale = 0.5 / ((double)nx * (double)nz);   // the forward x-transform's values are doubled
   if (launch_spec_thomas(spec, dscr, cpr, inv, yr, g, scale, !dir, s) != cudaSuccess) return PNP_ERR_CUDA;
   if (launch_fft_z<double>(spec, tz, g, true, s) != cudaSuccess) return PNP_ERR_CUDA;
   if (launch_fft_x_inv<double, double>(PoissonDst::Plain, spec, g, m, tx, tp, 0.0, x_dev, s) != cudaSuccess)

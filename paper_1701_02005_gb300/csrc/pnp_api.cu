@@ -799,7 +799,7 @@ cudaError_t spectral_solve(pnp_ctx* c, cplx<T>* spec, const cplx<T>* twz, bool n
   cudaError_t e = launch_fft_z<T>(spec, twz, c->g, false, st);
   if (e != cudaSuccess) return e;
   mark(c, st, neumann ? PNP_SITE_P_FFTZ : PNP_SITE_E_FFTZ);
-  const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
+  const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
   if constexpr (sizeof(T) == sizeof(float))
     e = launch_spec_thomas_df(spec, dscr, spec_df(c, neumann), yrows(c, neumann), c->g, scale, neumann, st);
   else
@@ -883,7 +883,7 @@ cudaError_t potential_mixed(pnp_ctx* c, cudaStream_t st, void* spec_buf, cplx<do
   e = launch_fft_z<float>(spec, twz, c->g, false, st);
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_FFTZ);
-  const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
+  const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
   const SpecMean mean = spec_mean(c);
   e = launch_spec_thomas_df(spec, dscr, spec_df(c, false), yrows(c, false), c->g, scale, false, st, &mean);
   if (e != cudaSuccess) return e;
@@ -938,7 +938,7 @@ cudaError_t potential_mixed_fp64(pnp_ctx* c, cudaStream_t st, void* spec_buf, cp
   e = launch_fft_z<double>(spec, twz, c->g, false, st);
   if (e != cudaSuccess) return e;
   mark(c, st, PNP_SITE_E_FFTZ);
-  const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
+  const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
   const SpecMean mean = spec_mean(c);
   e = launch_spec_thomas(spec, dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale, false, st, &mean);
   if (e != cudaSuccess) return e;
@@ -2074,7 +2074,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
   }
   c->g.lc_cn = pick[1];
   // 3: spectral y-solve (columns in shared memory or streamed), 4: z-transform threads per column
-  const double scale = 1.0 / ((double)c->g.nx * (double)c->g.nz);
+  const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
   for (int T : {16, 32}) {   // (FP64 has the streamed form only)
     c->g.lc_spec = T;
     float t = time_launches(c, [&] {

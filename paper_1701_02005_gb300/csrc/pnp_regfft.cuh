@@ -9,9 +9,9 @@
 // memory the G-point DFTs over g run in registers again.  One shared-memory
 // round trip per transform instead of one per radix-4 stage.
 //
-// The small DFTs are radix-2 decimation in frequency, unrolled by template
-// recursion so that every twiddle is a compile-time constant; the constants
-// come from a Taylor series of sin and cos on [0, pi/4] (octant symmetry),
+// The small DFTs are radix-2 (decimation in time in FP64, in frequency in FP32),
+// unrolled by template recursion so that every twiddle is a compile-time constant;
+// the constants come from a Taylor series of sin and cos on [0, pi/4] (octant symmetry),
 // written here from the series itself and evaluated by the compiler.
 #pragma once
 
@@ -128,10 +128,66 @@ __host__ __device__ __forceinline__ void dif_stages(cplx<T>* v) {
   }
 }
 
+// The butterfly a, c -> a + w c, a - w c with w = W_M^I (forward) or its conjugate
+// (inverse), in the precision T of the transform.  A general w costs six fused
+// multiply-adds (Linzer & Feig 1993): with tau the smaller of sin/cos and cos/sin,
+// w c = cos (1 + i tau) c or sin (tau + i) c, two for the bracket and one for each
+// of the four sums; W^0 and W^{M/4} cost four additions.
+template <bool INV, int I, int M, typename T>
+__host__ __device__ __forceinline__ void butterfly(cplx<T>& a, cplx<T>& c) {
+  cplx<T> t = c;
+  if constexpr (I == 0 || 4 * I == M) {
+    if constexpr (I != 0) t = INV ? cplx<T>{-c.y, c.x} : cplx<T>{c.y, -c.x};
+    const cplx<T> b = a;
+    a = cadd(b, t);
+    c = csub(b, t);
+  } else {
+    constexpr double cs = cos2pi(I, M), sn = (INV ? 1.0 : -1.0) * sin2pi(I, M);
+    constexpr bool by_cos = (cs < 0 ? -cs : cs) >= (sn < 0 ? -sn : sn);
+    constexpr T f = (T)(by_cos ? cs : sn), tau = (T)(by_cos ? sn / cs : cs / sn);
+    if constexpr (by_cos) t = {c.x - tau * c.y, c.y + tau * c.x};
+    else t = {tau * c.x - c.y, tau * c.y + c.x};
+    const cplx<T> b = a;
+    a = {b.x + f * t.x, b.y + f * t.y};
+    c = {b.x - f * t.x, b.y - f * t.y};
+  }
+}
+
+// Decimation in time over the bit-reversed order of v: element p of the reordered
+// array is v[bitrev(p)].
+template <bool INV, int M, int HALF, int B, int I, typename T>
+__host__ __device__ __forceinline__ void dit_block(cplx<T>* v) {
+  if constexpr (I < HALF) {
+    butterfly<INV, I, 2 * HALF>(v[bitrev(B + I, M)], v[bitrev(B + I + HALF, M)]);
+    dit_block<INV, M, HALF, B, I + 1>(v);
+  }
+}
+
+template <bool INV, int M, int HALF, int B, typename T>
+__host__ __device__ __forceinline__ void dit_blocks(cplx<T>* v) {
+  if constexpr (B < M) {
+    dit_block<INV, M, HALF, B, 0>(v);
+    dit_blocks<INV, M, HALF, B + 2 * HALF>(v);
+  }
+}
+
+template <bool INV, int M, int HALF, typename T>
+__host__ __device__ __forceinline__ void dit_stages(cplx<T>* v) {
+  if constexpr (HALF < M) {
+    dit_blocks<INV, M, HALF, 0>(v);
+    dit_stages<INV, M, 2 * HALF>(v);
+  }
+}
+
 // In-place M-point DFT of v[0..M); the result X[k] is left at v[bitrev(k, M)].
+// FP64 in time: the FP64 pipe is the bound and 16 points take 148 operations
+// against 168 in frequency (z-transform, 128x97x128: 55.3 -> 53.2 us).  FP32 in
+// frequency: memory and latency bound it and fewer operations gain nothing
+// (256x193x256: 25.2 against 26.1 us).
 template <bool INV, int M, typename T>
 __host__ __device__ __forceinline__ void dft(cplx<T>* v) {
-  dif_stages<INV, M, M / 2>(v);
+  if constexpr (sizeof(T) == 8) dit_stages<INV, M, 1>(v);
+  else dif_stages<INV, M, M / 2>(v);
 }
 
 // f(std::integral_constant<int, I>) for I = B .. E-1: a loop whose index is a
