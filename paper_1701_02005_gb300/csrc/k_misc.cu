@@ -582,50 +582,35 @@ template cudaError_t launch_init_fields<float>(const Fields<float>&, const Geo&,
                                                double, double, uint64_t, double, const double*, cudaStream_t);
 // ---------------------------------------------------------------------------
 // Wall potentials that vary along the walls (the walls may carry any
-// potential): Phi = V y + off + lift + phi, lift = Phi_0' + psi with psi the
-// homogeneous-Dirichlet solution of L psi = -(d_xx + d_zz) Phi_0'.
+// potential): Phi = V y + off + lift + phi, lift the charge-free potential between
+// the walls' variations.
 // ---------------------------------------------------------------------------
-__global__ void k_wall_lift_source(double* __restrict__ src, const double* __restrict__ B,
-                                   const double* __restrict__ T, const double* __restrict__ yc, Geo g) {
-  const size_t P = (size_t)g.nz * g.nx, n = (size_t)g.nyc * P;
-  for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(c / P);
-    const int r = (int)(c - (size_t)j * P), k = r / g.nx, i = r - k * g.nx;
-    const int ip = i + 1 == g.nx ? 0 : i + 1, im = i == 0 ? g.nx - 1 : i - 1;
-    const int kp = k + 1 == g.nz ? 0 : k + 1, km = k == 0 ? g.nz - 1 : k - 1;
-    auto lap = [&](const double* q) {
-      const double q0 = q[r];
-      return (q[k * g.nx + ip] - 2.0 * q0 + q[k * g.nx + im]) * g.idx * g.idx +
-             (q[kp * g.nx + i] - 2.0 * q0 + q[km * g.nx + i]) * g.idz * g.idz;
-    };
-    src[c] = -(0.5 * (1.0 - yc[j]) * lap(B) + 0.5 * (1.0 + yc[j]) * lap(T));
-  }
+// What the wall values leave on the right of the first and last cell planes' rows.
+__global__ void k_wall_rows(double* __restrict__ src, const double* __restrict__ B, const double* __restrict__ T,
+                            double Bm, double Tm, double cb, double ct, int P) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= P) return;
+  src[r] = cb * (B[r] - Bm);
+  src[P + r] = ct * (T[r] - Tm);
 }
 
-__global__ void k_wall_lift_finish(double* __restrict__ lift64, float* __restrict__ lift32,
-                                   const double* __restrict__ B, const double* __restrict__ T, double Bm, double Tm,
-                                   double off, const double* __restrict__ yc, Geo g) {
-  const size_t P = (size_t)g.nz * g.nx, n = (size_t)g.nyc * P;
-  for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(c / P);
-    const size_t r = c - (size_t)j * P;
-    const double v = lift64[c] + 0.5 * (1.0 - yc[j]) * (B[r] - Bm) + 0.5 * (1.0 + yc[j]) * (T[r] - Tm);
-    lift32[c] = (float)v;
-    lift64[c] = v + off;
-  }
-}
-
-cudaError_t launch_wall_lift_source(double* src, const double* B, const double* T, double Bm, double Tm,
-                                    const double* yc, const Geo& g, cudaStream_t s) {
-  (void)Bm;
-  (void)Tm;   // the x/z second differences of a constant vanish
-  k_wall_lift_source<<<1216, 256, 0, s>>>(src, B, T, yc, g);
+cudaError_t launch_wall_rows(double* src, const double* B, const double* T, double Bm, double Tm, double cb, double ct,
+                             const Geo& g, cudaStream_t s) {
+  const int P = g.nz * g.nx;
+  k_wall_rows<<<(P + 255) / 256, 256, 0, s>>>(src, B, T, Bm, Tm, cb, ct, P);
   return cudaGetLastError();
 }
 
-cudaError_t launch_wall_lift_finish(double* lift64, float* lift32, const double* B, const double* T, double Bm,
-                                    double Tm, double off, const double* yc, const Geo& g, cudaStream_t s) {
-  k_wall_lift_finish<<<1216, 256, 0, s>>>(lift64, lift32, B, T, Bm, Tm, off, yc, g);
+__global__ void k_lift_copy(double* __restrict__ lift64, float* __restrict__ lift32, double off, size_t n) {
+  const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n) return;
+  const double v = lift64[c];
+  lift32[c] = (float)v;
+  if (off != 0.0) lift64[c] = v + off;
+}
+
+cudaError_t launch_lift_copy(double* lift64, float* lift32, double off, size_t n, cudaStream_t s) {
+  k_lift_copy<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(lift64, lift32, off, n);
   return cudaGetLastError();
 }
 

@@ -14,6 +14,8 @@
 // c+ <-> c-, Phi -> -Phi, under which the plane Couette problem is invariant,
 // so that one network serves both walls.  Streamwise velocities are taken
 // relative to the wall: u_rel = u + Uw (bottom), Uw - u (top).
+#include <cooperative_groups.h>
+
 #include "pnp_common.cuh"
 #include "pnp_wall.cuh"
 
@@ -62,28 +64,37 @@ __global__ void k_restrict_v(const T* __restrict__ f, WallMap wm, double* __rest
 }
 
 // Feature rows: [wall][k][i] x [field][d], d = 0..ncells-1 cells away from the wall.
+// A block forms 32 rows, one thread per row and cell, and writes them out
+// contiguously from shared memory (128x49x128, 8 cells: XX us, 22 us with a thread
+// per row storing its 40 values 160 bytes apart).
+constexpr int kFeatRows = 32;
+
 template <typename TV>
-__global__ void k_wall_features(const TV* __restrict__ u, const TV* __restrict__ w, IonView ions,
-                                const double* __restrict__ yc, Geo g, double V, double Uw, int ncells,
-                                const double* __restrict__ lift, float* __restrict__ X) {
-  const size_t P = (size_t)g.nz * g.nx;
-  const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= 2 * P) return;
-  const int wall = (int)(r / P);
-  const size_t col = r - (size_t)wall * P;
-  float* row = X + r * (size_t)(5 * ncells);
-  for (int d = 0; d < ncells; ++d) {
+__global__ void __launch_bounds__(kFeatRows * 8)
+    k_wall_features(const TV* __restrict__ u, const TV* __restrict__ w, IonView ions, const double* __restrict__ yc,
+                    Geo g, double V, double Uw, int ncells, const double* __restrict__ lift, float* __restrict__ X) {
+  __shared__ float sh[kFeatRows][41];
+  const size_t P = (size_t)g.nz * g.nx, r0 = (size_t)blockIdx.x * kFeatRows;
+  const int t = threadIdx.x, d = threadIdx.y, nf = 5 * ncells;
+  const size_t r = r0 + t;
+  if (r < 2 * P && d < ncells) {
+    const int wall = (int)(r >= P);
+    const size_t col = r - (wall ? P : 0);
     const int j = wall == 0 ? d : g.nyc - 1 - d;
     const size_t o = (size_t)j * P + col;
     const double phi = ions.phv(j, o) - V * yc[j] - (lift ? lift[o] : 0.0);
     const double ur = wall == 0 ? (double)u[o] + Uw : Uw - (double)u[o];
     const double cpo = ions.cpv(j, o), cmo = ions.cmv(j, o);
-    row[0 * ncells + d] = (float)ur;
-    row[1 * ncells + d] = (float)(double)w[o];
-    row[2 * ncells + d] = (float)(wall == 0 ? cpo : cmo);
-    row[3 * ncells + d] = (float)(wall == 0 ? cmo : cpo);
-    row[4 * ncells + d] = (float)(wall == 0 ? phi : -phi);
+    sh[t][0 * ncells + d] = (float)ur;
+    sh[t][1 * ncells + d] = (float)(double)w[o];
+    sh[t][2 * ncells + d] = (float)(wall == 0 ? cpo : cmo);
+    sh[t][3 * ncells + d] = (float)(wall == 0 ? cmo : cpo);
+    sh[t][4 * ncells + d] = (float)(wall == 0 ? phi : -phi);
   }
+  __syncthreads();
+  const int rows = (int)min((size_t)kFeatRows, 2 * P - r0);
+  float* out = X + r0 * nf;
+  for (int e = d * kFeatRows + t; e < rows * nf; e += kFeatRows * 8) out[e] = sh[e / nf][e % nf];
 }
 
 // Labels of coarse wall column (wall, kc, ic) from the fine state:
@@ -209,43 +220,61 @@ __global__ void k_relax_rates(float* __restrict__ Y, float* __restrict__ prev, i
 
 // Plane means of the two wall-shear-rate columns of each wall's rows (rows
 // [0, P) bottom, [P, 2P) top) over the rows with finite predictions, written
-// back to every row of that wall.
-__global__ void k_mean_rates(float* __restrict__ Y, int P) {
-  __shared__ float sh[3][256];
-  const int wall = blockIdx.x;
-  float a = 0.f, b = 0.f, n = 0.f;
-  for (int r = threadIdx.x; r < P; r += blockDim.x) {
-    const float ya = Y[(size_t)(wall * P + r) * 5 + 0], yb = Y[(size_t)(wall * P + r) * 5 + 1];
+// back to every row of that wall.  A cluster of eight blocks per wall: each sums
+// its share, then adds up all eight blocks' sums through distributed shared memory
+// (the same order in every block).  32,768 rows: XX us; 39 us with one block per
+// wall, bound by the latency of its 64 passes over the rows.
+constexpr int kMeanCta = 8, kMeanThreads = 512;
+
+__global__ void __cluster_dims__(kMeanCta, 1, 1) __launch_bounds__(kMeanThreads) k_mean_rates(float* __restrict__ Y, int P) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ float sh[3][kMeanThreads / 32], tot[3];
+  const int wall = blockIdx.y, rank = (int)cl.block_rank(), t = threadIdx.x, warp = t >> 5;
+  float* y = Y + (size_t)wall * P * 5;
+  float v[3] = {0.f, 0.f, 0.f};
+#pragma unroll 4
+  for (int r = rank * kMeanThreads + t; r < P; r += kMeanCta * kMeanThreads) {
+    const float ya = y[(size_t)r * 5 + 0], yb = y[(size_t)r * 5 + 1];
     if (isfinite(ya) && isfinite(yb)) {   // a non-finite prediction does not enter the mean
-      a += ya;
-      b += yb;
-      n += 1.f;
+      v[0] += ya;
+      v[1] += yb;
+      v[2] += 1.f;
     }
   }
-  sh[0][threadIdx.x] = a;
-  sh[1][threadIdx.x] = b;
-  sh[2][threadIdx.x] = n;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if ((t & 31) == 0) sh[q][warp] = v[q];
+  }
   __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      sh[0][threadIdx.x] += sh[0][threadIdx.x + st];
-      sh[1][threadIdx.x] += sh[1][threadIdx.x + st];
-      sh[2][threadIdx.x] += sh[2][threadIdx.x + st];
-    }
-    __syncthreads();
+  if (t < 3) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < kMeanThreads / 32; ++i) s += sh[t][i];
+    tot[t] = s;
   }
+  cl.sync();
+  float m[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int b = 0; b < kMeanCta; ++b) {
+    const float* o = cl.map_shared_rank(tot, b);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) m[q] += o[q];
+  }
+  cl.sync();   // no block leaves while its sums are read
   // no finite row: NaN, which the wall-value kernel turns into the no-slip wall
-  const float cnt = sh[2][0];
-  const float ma = cnt > 0.f ? sh[0][0] / cnt : __int_as_float(0x7fc00000);
-  const float mb = cnt > 0.f ? sh[1][0] / cnt : __int_as_float(0x7fc00000);
-  for (int r = threadIdx.x; r < P; r += blockDim.x) {
-    Y[(size_t)(wall * P + r) * 5 + 0] = ma;
-    Y[(size_t)(wall * P + r) * 5 + 1] = mb;
+  const float ma = m[2] > 0.f ? m[0] / m[2] : __int_as_float(0x7fc00000);
+  const float mb = m[2] > 0.f ? m[1] / m[2] : __int_as_float(0x7fc00000);
+  for (int r = rank * kMeanThreads + t; r < P; r += kMeanCta * kMeanThreads) {
+    y[(size_t)r * 5 + 0] = ma;
+    y[(size_t)r * 5 + 1] = mb;
   }
 }
 
 cudaError_t launch_mean_rates(float* Y, int P, cudaStream_t s) {
-  k_mean_rates<<<2, 256, 0, s>>>(Y, P);
+  k_mean_rates<<<dim3(kMeanCta, 2), kMeanThreads, 0, s>>>(Y, P);
   return cudaGetLastError();
 }
 
@@ -367,7 +396,8 @@ template <typename TV>
 cudaError_t launch_wall_features(const TV* u, const TV* w, const IonView& ions, const double* yc, const Geo& g,
                                  double V, double Uw, int ncells, const double* lift, float* X, cudaStream_t s) {
   const size_t n = 2 * (size_t)g.nz * g.nx;
-  k_wall_features<TV><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(u, w, ions, yc, g, V, Uw, ncells, lift, X);
+  k_wall_features<TV><<<(unsigned)((n + kFeatRows - 1) / kFeatRows), dim3(kFeatRows, 8), 0, s>>>(u, w, ions, yc, g, V,
+                                                                                              Uw, ncells, lift, X);
   return cudaGetLastError();
 }
 

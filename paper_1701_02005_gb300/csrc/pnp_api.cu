@@ -952,6 +952,45 @@ cudaError_t potential_mixed_fp64(pnp_ctx* c, cudaStream_t st, void* spec_buf, cp
   return e;
 }
 
+// The charge-free potential lift of wall potentials that vary along the walls (B, T
+// less their means Bm, Tm): (d_xx + d_zz + L_y) lift = 0 between those walls.  The
+// wall values enter the y-operator's first and last rows only, so the forward
+// transforms run on two planes; the solve, and the transforms back, as in every FP64
+// Dirichlet solve (the scratch of the pressure pipeline).  lift32: the FP32 copy
+// without off, lift64: with it.  One solve of 128x49x128: 97 us, 201 us with the
+// linear lift's x/z curvature as the source on every plane.
+cudaError_t lift_solve(pnp_ctx* c, double Bm, double Tm, double off) {
+  const Metrics m = metrics(c);
+  const cplx<double>* twx = (const cplx<double>*)c->twx_d;
+  const cplx<double>* twp = (const cplx<double>*)c->twp_d;
+  const cplx<double>* twz = (const cplx<double>*)c->twz_d;
+  cplx<double>* spec = (cplx<double>*)c->spec;
+  cplx<double>* walls = c->dscr;   // [2 planes], before the solve's forward values need it
+  const int n = c->g.nyc;
+  const size_t Ps = (size_t)c->g.nz * c->g.mp;
+  Geo g2 = c->g;
+  g2.nyc = 2;
+  cudaStream_t s = c->stream;
+  cudaError_t e = launch_wall_rows(c->sreal, c->wallB_d, c->wallT_d, Bm, Tm, -1.0 / (c->h[0] * c->dy[0]),
+                                   -1.0 / (c->h[n] * c->dy[n - 1]), c->g, s);
+  if (e == cudaSuccess)
+    e = launch_fft_x_fwd<double, double>(PoissonSrc::Plain, nullptr, nullptr, nullptr, nullptr, nullptr, c->sreal, 1.0,
+                                         g2, m, walls, twx, twp, s);
+  if (e == cudaSuccess) e = launch_fft_z<double>(walls, twz, g2, false, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(spec, 0, sizeof(cplx<double>) * Ps * n, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(spec, walls, sizeof(cplx<double>) * Ps, cudaMemcpyDeviceToDevice, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(spec + Ps * (n - 1), walls + Ps, sizeof(cplx<double>) * Ps, cudaMemcpyDeviceToDevice, s);
+  const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
+  if (e == cudaSuccess)
+    e = launch_spec_thomas(spec, c->dscr, c->spc_cprD, c->spc_invD, yrows(c, false), c->g, scale, false, s);
+  if (e == cudaSuccess) e = launch_fft_z<double>(spec, twz, c->g, true, s);
+  if (e == cudaSuccess)
+    e = launch_fft_x_inv<double, double>(PoissonDst::Plain, spec, c->g, m, twx, twp, 0.0, c->lift64, s);
+  if (e == cudaSuccess) e = launch_lift_copy(c->lift64, c->lift32, off, c->nc, s);
+  return e;
+}
+
 // FP64 scratch of the FP64-arithmetic CN solves: the FP64 copies of the ion
 // state, Phi, H_c+- and the conversion stage are not read during a mixed step
 // (they are materialised on demand afterwards), so they hold the forward values.
@@ -1587,20 +1626,8 @@ int pnp_set_wall_potential(pnp_ctx* c, const double* bottom, const double* top) 
     const double Bm = sb / (double)P, Tm = st / (double)P;
     CK(cudaMemcpyAsync(c->wallB_d, bottom, sizeof(double) * P, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->wallT_d, top, sizeof(double) * P, cudaMemcpyHostToDevice, c->stream));
-    // lift = Phi_0' + psi: the charge-free potential of the zero-mean wall
-    // variations, one FP64 Dirichlet solve (the scratch of the pressure pipeline)
-    const Metrics m = metrics(c);
-    cplx<double>* spec = (cplx<double>*)c->spec;
-    const cplx<double>* twx = (const cplx<double>*)c->twx_d;
-    const cplx<double>* twp = (const cplx<double>*)c->twp_d;
-    const cplx<double>* twz = (const cplx<double>*)c->twz_d;
-    CK(launch_wall_lift_source(c->sreal, c->wallB_d, c->wallT_d, Bm, Tm, c->yc_d, c->g, c->stream));
-    CK(launch_fft_x_fwd<double, double>(PoissonSrc::Plain, nullptr, nullptr, nullptr, nullptr, nullptr, c->sreal, 1.0,
-                                        c->g, m, spec, twx, twp, c->stream));
-    CK(spectral_solve<double>(c, spec, twz, false));
-    CK(launch_fft_x_inv<double, double>(PoissonDst::Plain, spec, c->g, m, twx, twp, 0.0, c->lift64, c->stream));
     const double off = 0.5 * (Tm + Bm);
-    CK(launch_wall_lift_finish(c->lift64, c->lift32, c->wallB_d, c->wallT_d, Bm, Tm, off, c->yc_d, c->g, c->stream));
+    CK(lift_solve(c, Bm, Tm, off));
     c->wall_map = true;
     c->wall_off = off;
     c->ph.V = 0.5 * (Tm - Bm);
@@ -2618,27 +2645,6 @@ int pnp_set_wallmodel_coupling(pnp_ctx* c, int mode, double relax) {
 }
 
 namespace {
-// Lift of the offset map: the charge-free potential of wall offsets B, T kept
-// with their plane means (relative to the uniform walls, so V and the constant
-// offset stay those of pnp_set_params).
-cudaError_t edl_lift(pnp_ctx* c) {
-  const Metrics m = metrics(c);
-  cplx<double>* spec = (cplx<double>*)c->spec;
-  const cplx<double>* twx = (const cplx<double>*)c->twx_d;
-  const cplx<double>* twp = (const cplx<double>*)c->twp_d;
-  const cplx<double>* twz = (const cplx<double>*)c->twz_d;
-  cudaError_t e = launch_wall_lift_source(c->sreal, c->wallB_d, c->wallT_d, 0.0, 0.0, c->yc_d, c->g, c->stream);
-  if (e == cudaSuccess)
-    e = launch_fft_x_fwd<double, double>(PoissonSrc::Plain, nullptr, nullptr, nullptr, nullptr, nullptr, c->sreal, 1.0,
-                                         c->g, m, spec, twx, twp, c->stream);
-  if (e == cudaSuccess) e = spectral_solve<double>(c, spec, twz, false);
-  if (e == cudaSuccess)
-    e = launch_fft_x_inv<double, double>(PoissonDst::Plain, spec, c->g, m, twx, twp, 0.0, c->lift64, c->stream);
-  if (e == cudaSuccess)
-    e = launch_wall_lift_finish(c->lift64, c->lift32, c->wallB_d, c->wallT_d, 0.0, 0.0, 0.0, c->yc_d, c->g, c->stream);
-  return e;
-}
-
 int edl_potential(pnp_ctx* c, const float* X, int ncells, const float* Y) {
   if (!c->have_state) return PNP_ERR_STATE;
   const size_t P = (size_t)c->g.nz * c->g.nx;
@@ -2656,7 +2662,7 @@ int edl_potential(pnp_ctx* c, const float* X, int ncells, const float* Y) {
   const double lim = std::max(1.0, std::fabs(c->ph.V));
   CK(launch_edl_offsets(X, ncells, Y, P, c->edl_phi_gain, lim, c->lift64, c->g.nyc, c->wallB_d, c->wallT_d,
                         c->stream));
-  CK(edl_lift(c));
+  CK(lift_solve(c, 0.0, 0.0, 0.0));   // the offsets keep their plane means: V stays that of pnp_set_params
   // the potential of the present ions under the moved walls: in a mixed context that
   // steps on its shadows, the step's own potential pipeline (writes phi')
   if (c->precision == PNP_MIXED && c->refs_valid) {
