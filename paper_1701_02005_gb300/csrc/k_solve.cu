@@ -474,14 +474,27 @@ __global__ void __launch_bounds__(256) k_fft_x_inv_reg(PoissonDst dst, const cpl
   });
 }
 
-// Rows per 128-thread block of the register x-transforms (smaller blocks share
+static int fft_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  return sms;
+}
+
+// Rows per block of the register x-transforms: 128 threads (smaller blocks share
 // the GPU better with the other stream: 2.583 against 2.593 ms per step with
-// 256 threads on the 256x193x256 workload), and shared memory.
-template <int NH, int R1>
-constexpr int fx_rows() { return 128 / (NH / R1); }
+// 256 threads on the 256x193x256 workload); in FP64, where few busy SMs means few
+// FP64 pipes, down to one warp until every SM has two blocks (32x33x32: 6.9
+// against 8.2 us; in FP32 the smaller blocks gain nothing).
+static int fx_rows(int G, int nrows, bool fp64) {
+  const int want = fp64 ? 2 * fft_sms() : 1;
+  int rows = 128 / G;
+  while (rows * G > 32 && (nrows + rows - 1) / rows < want) rows >>= 1;
+  return rows;
+}
 template <int NH, int R1, typename T>
-constexpr size_t fx_smem() {
-  return sizeof(cplx<T>) * ((size_t)2 * NH + 1 + (size_t)fx_rows<NH, R1>() * fx_row_stride<NH, R1>());
+constexpr size_t fx_smem(int rows) {
+  return sizeof(cplx<T>) * ((size_t)2 * NH + 1 + (size_t)rows * fx_row_stride<NH, R1>());
 }
 
 template <typename T>
@@ -506,22 +519,23 @@ cudaError_t launch_fft_x_fwd(PoissonSrc kind, const TV* u, const TV* v, const TV
   SrcArgs<T, TV> a{kind, u, v, w, cp, cm, plain, scale, sa, sb, (T)(scale * g.idx), (T)(scale * g.idz), idyT,
                    (T)scale, la, lb};
   {
-    auto go = [&](auto kern, int G, int rows, size_t smem) {
+    auto go = [&](auto kern, int G, size_t (*smem_of)(int)) {
+      const int nrows = g.nyc * g.nz, rows = fx_rows(G, nrows, sizeof(T) == 8);
+      const size_t smem = smem_of(rows);
       if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
       }
-      const int nrows = g.nyc * g.nz;
       kern<<<(nrows + rows - 1) / rows, dim3(G, rows), smem, s>>>(a, g, m, spec, tw_half, tw_post);
       return cudaGetLastError();
     };
     switch (g.nx / 2) {
-      case 16: return go(k_fft_x_fwd_reg<16, 4, T, TV>, 4, fx_rows<16, 4>(), fx_smem<16, 4, T>());
-      case 32: return go(k_fft_x_fwd_reg<32, 8, T, TV>, 4, fx_rows<32, 8>(), fx_smem<32, 8, T>());
-      case 64: return go(k_fft_x_fwd_reg<64, 8, T, TV>, 8, fx_rows<64, 8>(), fx_smem<64, 8, T>());
-      case 128: return go(k_fft_x_fwd_reg<128, 16, T, TV>, 8, fx_rows<128, 16>(), fx_smem<128, 16, T>());
-      case 256: return go(k_fft_x_fwd_reg<256, 16, T, TV>, 16, fx_rows<256, 16>(), fx_smem<256, 16, T>());
-      case 512: return go(k_fft_x_fwd_reg<512, 32, T, TV>, 16, fx_rows<512, 32>(), fx_smem<512, 32, T>());
+      case 16: return go(k_fft_x_fwd_reg<16, 4, T, TV>, 4, fx_smem<16, 4, T>);
+      case 32: return go(k_fft_x_fwd_reg<32, 8, T, TV>, 4, fx_smem<32, 8, T>);
+      case 64: return go(k_fft_x_fwd_reg<64, 8, T, TV>, 8, fx_smem<64, 8, T>);
+      case 128: return go(k_fft_x_fwd_reg<128, 16, T, TV>, 8, fx_smem<128, 16, T>);
+      case 256: return go(k_fft_x_fwd_reg<256, 16, T, TV>, 16, fx_smem<256, 16, T>);
+      case 512: return go(k_fft_x_fwd_reg<512, 32, T, TV>, 16, fx_smem<512, 32, T>);
       default: break;
     }
   }
@@ -594,23 +608,24 @@ cudaError_t launch_fft_x_inv(PoissonDst dst, const cplx<T>* spec, const Geo& g, 
                              const cplx<T>* tw_half, const cplx<T>* tw_post, double V, TO* out,
                              cudaStream_t s, const double* plane_add, const TO* cell_add) {
   {
-    auto go = [&](auto kern, int G, int rows, size_t smem) {
+    auto go = [&](auto kern, int G, size_t (*smem_of)(int)) {
+      const int nrows = g.nyc * g.nz, rows = fx_rows(G, nrows, sizeof(T) == 8);
+      const size_t smem = smem_of(rows);
       if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
       }
-      const int nrows = g.nyc * g.nz;
       kern<<<(nrows + rows - 1) / rows, dim3(G, rows), smem, s>>>(dst, spec, g, m, tw_half, tw_post, V, out, plane_add,
                                                                   cell_add);
       return cudaGetLastError();
     };
     switch (g.nx / 2) {
-      case 16: return go(k_fft_x_inv_reg<16, 4, T, TO>, 4, fx_rows<16, 4>(), fx_smem<16, 4, T>());
-      case 32: return go(k_fft_x_inv_reg<32, 8, T, TO>, 4, fx_rows<32, 8>(), fx_smem<32, 8, T>());
-      case 64: return go(k_fft_x_inv_reg<64, 8, T, TO>, 8, fx_rows<64, 8>(), fx_smem<64, 8, T>());
-      case 128: return go(k_fft_x_inv_reg<128, 16, T, TO>, 8, fx_rows<128, 16>(), fx_smem<128, 16, T>());
-      case 256: return go(k_fft_x_inv_reg<256, 16, T, TO>, 16, fx_rows<256, 16>(), fx_smem<256, 16, T>());
-      case 512: return go(k_fft_x_inv_reg<512, 32, T, TO>, 16, fx_rows<512, 32>(), fx_smem<512, 32, T>());
+      case 16: return go(k_fft_x_inv_reg<16, 4, T, TO>, 4, fx_smem<16, 4, T>);
+      case 32: return go(k_fft_x_inv_reg<32, 8, T, TO>, 4, fx_smem<32, 8, T>);
+      case 64: return go(k_fft_x_inv_reg<64, 8, T, TO>, 8, fx_smem<64, 8, T>);
+      case 128: return go(k_fft_x_inv_reg<128, 16, T, TO>, 8, fx_smem<128, 16, T>);
+      case 256: return go(k_fft_x_inv_reg<256, 16, T, TO>, 16, fx_smem<256, 16, T>);
+      case 512: return go(k_fft_x_inv_reg<512, 32, T, TO>, 16, fx_smem<512, 32, T>);
       default: break;
     }
   }
@@ -707,9 +722,15 @@ __global__ void __launch_bounds__(TM*(N / R1)) k_fft_z_reg(cplx<T>* __restrict__
   }
 }
 
+// TM columns per block; in FP64 one warp's worth where TM leaves fewer blocks than
+// SMs (128x49x128: 23.9 against 27.7 us, its two wall planes 14.5 against 26.8 us; in
+// FP32 the narrower rows of a plane lose: 7.1 against 4.6 us).
 template <int N, int R1, int TM, typename T>
 cudaError_t launch_fft_z_reg(cplx<T>* spec, const cplx<T>* tw, const Geo& g, bool inverse, cudaStream_t s) {
   constexpr int G = N / R1;
+  if constexpr (sizeof(T) == 8 && TM * G > 32)
+    if ((g.mh + TM - 1) / TM * g.nyc < fft_sms())
+      return launch_fft_z_reg<N, R1, 32 / G, T>(spec, tw, g, inverse, s);
   const size_t smem = sizeof(cplx<T>) * ((size_t)TM * (N + 1) + N);
   const dim3 grd((unsigned)((g.mh + TM - 1) / TM), (unsigned)g.nyc);
   auto go = [&](auto kern) {

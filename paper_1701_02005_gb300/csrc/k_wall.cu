@@ -65,7 +65,7 @@ __global__ void k_restrict_v(const T* __restrict__ f, WallMap wm, double* __rest
 
 // Feature rows: [wall][k][i] x [field][d], d = 0..ncells-1 cells away from the wall.
 // A block forms 32 rows, one thread per row and cell, and writes them out
-// contiguously from shared memory (128x49x128, 8 cells: XX us, 22 us with a thread
+// contiguously from shared memory (128x49x128, 8 cells: 13.5 us, 22 us with a thread
 // per row storing its 40 values 160 bytes apart).
 constexpr int kFeatRows = 32;
 
@@ -222,7 +222,7 @@ __global__ void k_relax_rates(float* __restrict__ Y, float* __restrict__ prev, i
 // [0, P) bottom, [P, 2P) top) over the rows with finite predictions, written
 // back to every row of that wall.  A cluster of eight blocks per wall: each sums
 // its share, then adds up all eight blocks' sums through distributed shared memory
-// (the same order in every block).  32,768 rows: XX us; 39 us with one block per
+// (the same order in every block).  32,768 rows: 5.5 us; 39 us with one block per
 // wall, bound by the latency of its 64 passes over the rows.
 constexpr int kMeanCta = 8, kMeanThreads = 512;
 
