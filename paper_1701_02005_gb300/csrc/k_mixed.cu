@@ -467,7 +467,10 @@ struct FusedArgs {
   size_t P;
 };
 
-template <bool ION>
+// PRE: a batch's row factors are loaded with its rows, before the stores of the
+// batch that they would otherwise wait behind; more registers (101 against 63 for
+// the ions), the same operations in the same order.
+template <bool ION, bool PRE>
 __global__ void __launch_bounds__(256) k_cn_backsub_fused(FusedArgs A, int fam0) {
   constexpr int CH = 8;
   const FusedFam& F = A.f[fam0 + blockIdx.y];
@@ -498,7 +501,8 @@ __global__ void __launch_bounds__(256) k_cn_backsub_fused(FusedArgs A, int fam0)
   int first = max(ch * jc - j0, 0);
   float dprev = ch > 0 ? dend[ch - 1] : 0.f;
   for (int jb = n - 1; jb >= 0; jb -= CH) {
-    float dd[CH], sh[CH], sl[CH];
+    float dd[CH], sh[CH], sl[CH], gg[CH], cc[CH];
+    float2 aa[CH];
 #pragma unroll
     for (int k = 0; k < CH; ++k)
       if (jb - k >= 0) {
@@ -506,6 +510,11 @@ __global__ void __launch_bounds__(256) k_cn_backsub_fused(FusedArgs A, int fam0)
         dd[k] = d[o];
         sh[k] = S[o];
         if (ION) sl[k] = L[o];
+        if (PRE) {
+          gg[k] = __ldg(F.G + jb - k);
+          cc[k] = __ldg(F.c + jb - k);
+          if (ION) aa[k] = __ldg(F.add + jb - k);
+        }
       }
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
@@ -516,10 +525,10 @@ __global__ void __launch_bounds__(256) k_cn_backsub_fused(FusedArgs A, int fam0)
           first = max(ch * jc - j0, 0);
           dprev = ch > 0 ? dend[ch - 1] : 0.f;
         }
-        x = fmaf(F.G[r], dprev, dd[k]) - F.c[r] * x;
+        x = fmaf(PRE ? gg[k] : F.G[r], dprev, dd[k]) - (PRE ? cc[k] : F.c[r]) * x;
         const size_t o = (size_t)r * P;
         if (ION) {
-          const float2 inc = F.add[r];
+          const float2 inc = PRE ? aa[k] : F.add[r];
           const dfl cv = df_add2(dfl{sh[k], sl[k]}, dfl{inc.x, inc.y}, x);
           S[o] = cv.h;
           L[o] = cv.l;
@@ -547,15 +556,21 @@ cudaError_t launch_mixed_cn_fused(const Fields<float>& f, const Shadows& sh, con
   A.f[4] = FusedFam{reinterpret_cast<const float*>(f.rcm), sh.cm, sh.cmL, R.dC_m + (size_t)l * g.nyc, ion.c, G.ion,
                     g.nyc, 0};
   const int T = g.lc_cn && g.lc_cn != 32 ? g.lc_cn : 128;
+  // the factors with the rows where every block of the heavier form is resident at
+  // once: ions and velocities in turn 27.9 against 30.2 us at 64x65x64, 48.3 against
+  // 56.4 at 128x97x128, 152 against 167 at 256x257x128; with more lines the blocks
+  // that no longer fit cost more than the loads (212 against 182 us at 256x193x256)
+  const bool pre = P <= 32768;
+  auto go = [&](auto kern, int fam0, unsigned nfam) {
+    kern<<<dim3((unsigned)((P + T - 1) / T), nfam, 1), T, 0, s>>>(A, fam0);
+    return cudaGetLastError();
+  };
   if (parts & kCnIons) {
-    k_cn_backsub_fused<true><<<dim3((unsigned)((P + T - 1) / T), 2, 1), T, 0, s>>>(A, 3);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = pre ? go(k_cn_backsub_fused<true, true>, 3, 2) : go(k_cn_backsub_fused<true, false>, 3, 2);
     if (e != cudaSuccess) return e;
   }
-  if (parts & kCnVelocity) {
-    k_cn_backsub_fused<false><<<dim3((unsigned)((P + T - 1) / T), 3, 1), T, 0, s>>>(A, 0);
-    return cudaGetLastError();
-  }
+  if (parts & kCnVelocity)
+    return pre ? go(k_cn_backsub_fused<false, true>, 0, 3) : go(k_cn_backsub_fused<false, false>, 0, 3);
   return cudaSuccess;
 }
 
