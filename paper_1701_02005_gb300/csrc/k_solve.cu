@@ -24,36 +24,43 @@ namespace pnp {
 // Crank-Nicolson y-solves.  One thread per (i, k) line; lines are consecutive
 // in x so every plane access is coalesced.  The matrix I - s L_y is the same
 // for every line, so its elimination factors (a, c, m) come precomputed.
+// One launch for all five families: a small grid's families run side by side and a
+// step has three launches fewer, a large one's share one last wave; the velocities
+// and the ions one after the other before.  Three 32x33x32 contexts in turn 97 ->
+// 92 us a step, 128x97x128 2865 -> 2831.  Blocks of 128 lines: of 32 and 64 lines 97
+// and 93 us, though a context alone takes 174.5 a step with those and 176.4 with 128.
 // ---------------------------------------------------------------------------
-template <typename TQ, typename TR>
-__global__ void k_cn_thomas(TQ* __restrict__ q0, TR* __restrict__ r0, TQ* __restrict__ q1,
-                            TR* __restrict__ r1, TQ* __restrict__ q2, TR* __restrict__ r2,
-                            CNRows rows0, CNRows rows1, CNRows rows2, int n0, int n1, int n2,
-                            int j00, int j01, int j02, size_t P) {
+struct CnFam {
+  double *q, *r;   // state and right-hand side at the family's first row
+  CNRows rows;
+  int n;
+};
+struct CnFams {
+  CnFam f[5];
+  size_t P;
+};
+
+__global__ void k_cn_thomas(const __grid_constant__ CnFams A) {
   constexpr int CH = 8;   // planes loaded ahead per sweep step
-  const size_t line = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t P = A.P, line = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (line >= P) return;
-  TQ* q;
-  TR* r;
-  CNRows rw;
-  int n, j0;
-  if (blockIdx.y == 0) { q = q0; r = r0; rw = rows0; n = n0; j0 = j00; }
-  else if (blockIdx.y == 1) { q = q1; r = r1; rw = rows1; n = n1; j0 = j01; }
-  else { q = q2; r = r2; rw = rows2; n = n2; j0 = j02; }
-  TR* rl = r + (size_t)j0 * P + line;
-  TQ* ql = q + (size_t)j0 * P + line;
+  const CnFam& F = A.f[blockIdx.y];
+  const CNRows rw = F.rows;
+  const int n = F.n;
+  double* rl = F.r + line;
+  double* ql = F.q + line;
   double d = 0.0;
   for (int jb = 0; jb < n; jb += CH) {
     double rr[CH];
 #pragma unroll
     for (int u = 0; u < CH; ++u)
-      if (jb + u < n) rr[u] = (double)rl[(size_t)(jb + u) * P];
+      if (jb + u < n) rr[u] = rl[(size_t)(jb + u) * P];
 #pragma unroll
     for (int u = 0; u < CH; ++u) {
       const int j = jb + u;
       if (j < n) {
         d = (rr[u] - rw.a[j] * d) * rw.m[j];
-        rl[(size_t)j * P] = (TR)d;
+        rl[(size_t)j * P] = d;
       }
     }
   }
@@ -63,34 +70,33 @@ __global__ void k_cn_thomas(TQ* __restrict__ q0, TR* __restrict__ r0, TQ* __rest
 #pragma unroll
     for (int u = 0; u < CH; ++u)
       if (jb - u >= 0) {
-        dd[u] = (double)rl[(size_t)(jb - u) * P];
-        qq[u] = (double)ql[(size_t)(jb - u) * P];
+        dd[u] = rl[(size_t)(jb - u) * P];
+        qq[u] = ql[(size_t)(jb - u) * P];
       }
 #pragma unroll
     for (int u = 0; u < CH; ++u) {
       const int j = jb - u;
       if (j >= 0) {
         x = dd[u] - rw.c[j] * x;
-        ql[(size_t)j * P] = (TQ)(qq[u] + x);
+        ql[(size_t)j * P] = qq[u] + x;
       }
     }
   }
 }
 
-template <typename TV>
-cudaError_t launch_cn_solves(const Fields<TV>& f, const Geo& g, const CNRows& vel, const CNRows& face,
+cudaError_t launch_cn_solves(const Fields<double>& f, const Geo& g, const CNRows& vel, const CNRows& face,
                              const CNRows& ion, cudaStream_t s) {
   const size_t P = (size_t)g.nz * g.nx;
   const int T = g.lc_cn ? g.lc_cn : 128;
-  dim3 grd((unsigned)((P + T - 1) / T), 3, 1);
-  // u, w: nyc cells from plane 0; v: the nyc-1 interior faces from plane 1
-  k_cn_thomas<TV, TV><<<grd, T, 0, s>>>(f.u, f.ru, f.v, f.rv, f.w, f.rw, vel, face, vel, g.nyc,
-                                        g.nyc - 1, g.nyc, 0, 1, 0, P);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  dim3 grd2((unsigned)((P + T - 1) / T), 2, 1);
-  k_cn_thomas<double, double><<<grd2, T, 0, s>>>(f.cp, f.rcp, f.cm, f.rcm, f.cm, f.rcm, ion, ion, ion,
-                                                 g.nyc, g.nyc, g.nyc, 0, 0, 0, P);
+  // u, w: nyc cells from plane 0; v: the nyc-1 interior faces from plane 1; all five
+  // families in one launch
+  const CnFams A{{{f.u, f.ru, vel, g.nyc},
+                  {f.v + P, f.rv + P, face, g.nyc - 1},
+                  {f.w, f.rw, vel, g.nyc},
+                  {f.cp, f.rcp, ion, g.nyc},
+                  {f.cm, f.rcm, ion, g.nyc}},
+                 P};
+  k_cn_thomas<<<dim3((unsigned)((P + T - 1) / T), 5, 1), T, 0, s>>>(A);
   return cudaGetLastError();
 }
 
@@ -1739,11 +1745,6 @@ cudaError_t launch_periodic_conv(const ConvArgs<T>& a, const Geo& g, cudaStream_
 
 template cudaError_t launch_periodic_conv<double>(const ConvArgs<double>&, const Geo&, cudaStream_t);
 template cudaError_t launch_periodic_conv<float>(const ConvArgs<float>&, const Geo&, cudaStream_t);
-
-template cudaError_t launch_cn_solves<double>(const Fields<double>&, const Geo&, const CNRows&, const CNRows&,
-                                              const CNRows&, cudaStream_t);
-template cudaError_t launch_cn_solves<float>(const Fields<float>&, const Geo&, const CNRows&, const CNRows&,
-                                             const CNRows&, cudaStream_t);
 
 template cudaError_t launch_fft_x_fwd<double, double>(PoissonSrc, const double*, const double*, const double*,
                                                       const double*, const double*, const double*, double,

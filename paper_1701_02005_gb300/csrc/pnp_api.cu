@@ -1020,25 +1020,22 @@ cudaError_t poisson_pair(pnp_ctx* c, double scale) {
   return e;
 }
 
-
-
-template <typename TV>
 cudaError_t substage(pnp_ctx* c, double dt, int l) {
   const Stage st{dt, kGam[l], kZet[l], kGam[l] + kZet[l], c->scheme == PNP_SCHEME_AF ? 1 : 0};
-  const Fields<TV> f = fields<TV>(c);
+  const Fields<double> f = fields<double>(c);
   mark(c, c->stream, -1);
-  cudaError_t e = launch_rhs<TV>(f, c->g, metrics(c), c->ph, st, c->stream);
+  cudaError_t e = launch_rhs<double>(f, c->g, metrics(c), c->ph, st, c->stream);
   if (e != cudaSuccess) return e;
   if (st.af) {
-    e = periodic_sweeps<double>(c, l, 3u, (double*)f.ru, (double*)f.rv, (double*)f.rw, f.rcp, f.rcm, c->stream);
+    e = periodic_sweeps<double>(c, l, 3u, f.ru, f.rv, f.rw, f.rcp, f.rcm, c->stream);
     if (e != cudaSuccess) return e;
   }
   mark(c, c->stream, PNP_SITE_RHS);
-  e = launch_cn_solves<TV>(f, c->g, cn_rows(c, l, c->wall_stress ? 3 : 0), cn_rows(c, l, 1), cn_rows(c, l, 2),
-                           c->stream);
+  e = launch_cn_solves(f, c->g, cn_rows(c, l, c->wall_stress ? 3 : 0), cn_rows(c, l, 1), cn_rows(c, l, 2),
+                       c->stream);
   if (e != cudaSuccess) return e;
   mark(c, c->stream, PNP_SITE_CN);
-  return poisson_pair<TV>(c, st.alp * dt);
+  return poisson_pair<double>(c, st.alp * dt);
 }
 
 // Mixed-precision substage (policy in k_mixed.cu).
@@ -1105,7 +1102,7 @@ cudaError_t substage_mixed(pnp_ctx* c, double dt, int l) {
 
 cudaError_t one_step(pnp_ctx* c, double dt) {
   for (int l = 0; l < 3; ++l) {
-    cudaError_t e = c->precision == PNP_FP64 ? substage<double>(c, dt, l) : substage_mixed(c, dt, l);
+    cudaError_t e = c->precision == PNP_FP64 ? substage(c, dt, l) : substage_mixed(c, dt, l);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1935,7 +1932,7 @@ int pnp_profile(pnp_ctx* c, int nsteps, double dt, double* ms_out, int nsites, i
   for (int n = 0; n < nsteps && rc == PNP_OK; ++n) {
     for (int l = 0; l < 3 && rc == PNP_OK; ++l) {
       prof.n = 0;
-      cudaError_t e = c->precision == PNP_FP64 ? substage<double>(c, dt, l) : substage_mixed(c, dt, l);
+      cudaError_t e = c->precision == PNP_FP64 ? substage(c, dt, l) : substage_mixed(c, dt, l);
       if (e != cudaSuccess || prof.n != PNP_PROFILE_SITES + 1 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         rc = PNP_ERR_CUDA;
         break;
@@ -1979,7 +1976,7 @@ int pnp_timeline(pnp_ctx* c, double dt, int in_graph, int cap, int* site_out, in
   cudaGraphExec_t exec = nullptr;
   if (in_graph && cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) rc = PNP_ERR_CUDA;
   for (int l = 0; l < 3 && rc == PNP_OK; ++l) {
-    cudaError_t e = c->precision == PNP_FP64 ? substage<double>(c, dt, l) : substage_mixed(c, dt, l);
+    cudaError_t e = c->precision == PNP_FP64 ? substage(c, dt, l) : substage_mixed(c, dt, l);
     if (e != cudaSuccess) rc = PNP_ERR_CUDA;
   }
   if (in_graph) {
@@ -2092,7 +2089,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
     c->g.lc_cn = T;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64)
-        launch_cn_solves<double>(fields<double>(c), c->g, cn_rows(c, 0, 0), cn_rows(c, 0, 1), cn_rows(c, 0, 2), c->stream);
+        launch_cn_solves(fields<double>(c), c->g, cn_rows(c, 0, 0), cn_rows(c, 0, 1), cn_rows(c, 0, 2), c->stream);
       else
         launch_mixed_cn(fields<float>(c), shadows(c), mixed_refs(c), c->g, cn_rows_f(c, 0, 0), cn_rows_f(c, 0, 1),
                         cn_rows_f(c, 0, 2), 0, kCnIons | kCnVelocity, c->stream);

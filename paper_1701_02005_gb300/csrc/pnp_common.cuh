@@ -143,8 +143,7 @@ template <typename TV>
 cudaError_t launch_rhs(const Fields<TV>& f, const Geo& g, const Metrics& m, const Phys& ph,
                        const Stage& st, cudaStream_t s);
 
-template <typename TV>
-cudaError_t launch_cn_solves(const Fields<TV>& f, const Geo& g, const CNRows& vel, const CNRows& face,
+cudaError_t launch_cn_solves(const Fields<double>& f, const Geo& g, const CNRows& vel, const CNRows& face,
                              const CNRows& ion, cudaStream_t s);
 
 // Poisson pipeline pieces.  Spectral buffer holds (nyc, nz, mp) complex T.
