@@ -678,12 +678,12 @@ __global__ void k_fft_z(cplx<T>* __restrict__ spec, const cplx<T>* __restrict__ 
 }
 
 // z-transform with the two-pass register FFT (pnp_regfft.cuh), FP32 or FP64: a block
-// owns TM consecutive m-columns of one y-plane; thread (tm, g) loads the
-// samples n = g + G r of column tm (TM-wide coalesced rows), does the R1-point
-// DFT in registers, multiplies by W_N^{g k1} and exchanges through shared
+// owns TM consecutive columns of all planes' Nx/2 + 1 each (DENSE) or of one y-plane;
+// thread (tm, g) loads the samples n = g + G r of column tm (TM-wide coalesced rows),
+// does the R1-point DFT in registers, multiplies by W_N^{g k1} and exchanges through shared
 // memory; thread g then does the G-point DFTs of its R1 / G values of k1 and
 // stores X[k1 + R1 k2].
-template <int N, int R1, int TM, bool INV, typename T>
+template <int N, int R1, int TM, bool INV, bool DENSE, typename T>
 __global__ void __launch_bounds__(TM*(N / R1)) k_fft_z_reg(cplx<T>* __restrict__ spec,
                                                            const cplx<T>* __restrict__ tw, Geo g) {
   constexpr int G = N / R1, PER = R1 / G;
@@ -697,9 +697,14 @@ __global__ void __launch_bounds__(TM*(N / R1)) k_fft_z_reg(cplx<T>* __restrict__
     if (INV) t.y = -t.y;
     twl[e] = t;
   }
-  const int m = blockIdx.x * TM + tm;
-  const bool live = m < g.mh;
-  cplx<T>* col = spec + (size_t)blockIdx.y * N * g.mp + (live ? m : 0);
+  int m = blockIdx.x * TM + tm, j = blockIdx.y;
+  bool live = m < g.mh;
+  if (DENSE) {
+    j = m / g.mh;
+    m -= j * g.mh;
+    live = j < g.nyc;
+  }
+  cplx<T>* col = spec + (live ? (size_t)j * N * g.mp + m : 0);
   cplx<T> v[R1];
 #pragma unroll
   for (int r = 0; r < R1; ++r) v[r] = live ? col[(size_t)(gi + G * r) * g.mp] : cplx<T>{T(0), T(0)};
@@ -728,17 +733,25 @@ __global__ void __launch_bounds__(TM*(N / R1)) k_fft_z_reg(cplx<T>* __restrict__
   }
 }
 
-// TM columns per block; in FP64 one warp's worth where TM leaves fewer blocks than
+// TM columns per block.  FP64: columns packed over the planes, 16 per block, since a
+// warp that holds the one column left over of a plane's Nx/2 + 1 takes as long on the
+// FP64 pipe as a full one, and since narrow blocks share out better (128x97x128: 53.2
+// us with 32 columns of one plane per block, 54.0 packed, 43.0 packed with 16; three
+// contexts in turn 2831 -> 2672 us a step).  FP32, bound by memory: by plane, whose
+// aligned rows win (256x193x256: 25.2 against 28.5 us packed; 1024x385x512: 481
+// against 590).  One warp's worth of columns in FP64 where TM leaves fewer blocks than
 // SMs (128x49x128: 23.9 against 27.7 us, its two wall planes 14.5 against 26.8 us; in
 // FP32 the narrower rows of a plane lose: 7.1 against 4.6 us).
 template <int N, int R1, int TM, typename T>
 cudaError_t launch_fft_z_reg(cplx<T>* spec, const cplx<T>* tw, const Geo& g, bool inverse, cudaStream_t s) {
   constexpr int G = N / R1;
   if constexpr (sizeof(T) == 8 && TM * G > 32)
-    if ((g.mh + TM - 1) / TM * g.nyc < fft_sms())
+    if ((g.mh * g.nyc + TM - 1) / TM < fft_sms())
       return launch_fft_z_reg<N, R1, 32 / G, T>(spec, tw, g, inverse, s);
   const size_t smem = sizeof(cplx<T>) * ((size_t)TM * (N + 1) + N);
-  const dim3 grd((unsigned)((g.mh + TM - 1) / TM), (unsigned)g.nyc);
+  constexpr bool DENSE = sizeof(T) == 8;
+  const dim3 grd = DENSE ? dim3((unsigned)((g.mh * g.nyc + TM - 1) / TM))
+                         : dim3((unsigned)((g.mh + TM - 1) / TM), (unsigned)g.nyc);
   auto go = [&](auto kern) {
     if (smem > 48 * 1024) {
       const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -747,18 +760,19 @@ cudaError_t launch_fft_z_reg(cplx<T>* spec, const cplx<T>* tw, const Geo& g, boo
     kern<<<grd, dim3(TM, G), smem, s>>>(spec, tw, g);
     return cudaGetLastError();
   };
-  return inverse ? go(k_fft_z_reg<N, R1, TM, true, T>) : go(k_fft_z_reg<N, R1, TM, false, T>);
+  return inverse ? go(k_fft_z_reg<N, R1, TM, true, DENSE, T>) : go(k_fft_z_reg<N, R1, TM, false, DENSE, T>);
 }
 
 template <typename T>
 cudaError_t launch_fft_z(cplx<T>* spec, const cplx<T>* tw_z, const Geo& g, bool inverse, cudaStream_t s) {
   // register transforms for 16 <= Nz <= 512 unless the stage-by-stage kernel is asked for
   if (g.lc_fftz_ty != 64) {
+    constexpr int W = sizeof(T) == 8 ? 16 : 32;
     switch (g.nz) {
-      case 16: return launch_fft_z_reg<16, 4, 32, T>(spec, tw_z, g, inverse, s);
-      case 32: return launch_fft_z_reg<32, 8, 32, T>(spec, tw_z, g, inverse, s);
-      case 64: return launch_fft_z_reg<64, 8, 32, T>(spec, tw_z, g, inverse, s);
-      case 128: return launch_fft_z_reg<128, 16, 32, T>(spec, tw_z, g, inverse, s);
+      case 16: return launch_fft_z_reg<16, 4, W, T>(spec, tw_z, g, inverse, s);
+      case 32: return launch_fft_z_reg<32, 8, W, T>(spec, tw_z, g, inverse, s);
+      case 64: return launch_fft_z_reg<64, 8, W, T>(spec, tw_z, g, inverse, s);
+      case 128: return launch_fft_z_reg<128, 16, W, T>(spec, tw_z, g, inverse, s);
       case 256: return launch_fft_z_reg<256, 16, 16, T>(spec, tw_z, g, inverse, s);
       case 512: return launch_fft_z_reg<512, 32, 8, T>(spec, tw_z, g, inverse, s);
       default: break;
