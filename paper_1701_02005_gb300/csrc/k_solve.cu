@@ -12,6 +12,7 @@
 // split into the N/2 + 1 non-negative frequencies.  Forward transforms carry
 // no normalisation and the real ones a factor 2; the spectral solve multiplies by
 // 1/(2 Nx Nz).
+#include <algorithm>
 #include <type_traits>
 
 #include "pnp_common.cuh"
@@ -853,166 +854,192 @@ __device__ __forceinline__ void sp_cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
-__device__ __forceinline__ void sp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void sp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-// all but the groups after number g of four, then one more
-__device__ __forceinline__ void sp_wait_group(int g) {
-  switch (g) {
-    case 0: sp_wait<4>(); break;
-    case 1: sp_wait<3>(); break;
-    case 2: sp_wait<2>(); break;
-    default: sp_wait<1>(); break;
-  }
-}
 constexpr int kSpRows = 4;   // rows per batch of loads
 
-// Rows per copy group of a sweep over `rows` rows, a multiple of the batch.
-__device__ __forceinline__ int sp_group_rows(int rows) {
-  return max(kSpRows, ((rows + 3) / 4 + kSpRows - 1) / kSpRows * kSpRows);
+// One row of the forward sweep, d <- r v - (o v) d (r: transform value, v: 1/pivot, o:
+// off-diagonal): the products with v do not wait for d, so the chain through d is one
+// df_add_mul.  Scalar and packed: the same bits.
+__device__ __forceinline__ dfl sp_scaled(float r, float2 v) {
+  const float xh = __fmul_rn(r, v.x);
+  return {xh, __fmaf_rn(r, v.y, __fmaf_rn(r, v.x, -xh))};
+}
+__device__ __forceinline__ dfl sp_forward(float r, float2 v, float2 o, dfl d) {
+  return df_add_mul(sp_scaled(r, v), df_mul(dfl{-o.x, -o.y}, dfl{v.x, v.y}), d);
+}
+__device__ __forceinline__ df2 sp_forward(float2 r, float2 v, float2 o, df2 d) {
+  const float2 vh = f2(v.x);
+  const float2 xh = __fmul2_rn(r, vh);
+  const float2 xl = __ffma2_rn(r, f2(v.y), __ffma2_rn(r, vh, __fmul2_rn(xh, f2(-1.f))));
+  return df2_add_mul(df2{xh, xl}, df_mul(dfl{-o.x, -o.y}, dfl{v.x, v.y}), d);
 }
 
-// Per row of 16 points: transform values, 1/pivot, cpr, and the two off-diagonals.
-constexpr size_t spec_smem_df(int n) { return (size_t)n * (3 * 16 * 8 + 2 * 8); }
+// The middle row, from the rows below (d) and above (du).
+__device__ __forceinline__ dfl sp_middle(float r, float2 v, float2 a, float2 c, dfl d, dfl du) {
+  const dfl x = df_add_mul(df_add_mul(dfl{r, 0.f}, dfl{-a.x, -a.y}, d), dfl{-c.x, -c.y}, du);
+  return df_mul(x, dfl{v.x, v.y});
+}
+__device__ __forceinline__ df2 sp_middle(float2 r, float2 v, float2 a, float2 c, df2 d, df2 du) {
+  const df2 x = df2_add_mul(df2_add_mul(df2{r, f2(0.f)}, dfl{-a.x, -a.y}, d), dfl{-c.x, -c.y}, du);
+  return df2_mul(x, dfl{v.x, v.y});
+}
 
-// Columns in shared memory, double-float.  A warp solves 16 consecutive spectral
-// points of the plane (n mp + m, padding columns included), both parts of a point
-// in one lane (packed FP32): lanes 0-15 eliminate from the bottom wall, lanes
-// 16-31 from the top wall.  Every load of the block is issued before the first
-// operation (cp.async: four groups of rows in sweep order and one for the back
-// substitution's factors), so a column costs one memory latency instead of one
-// per batch of rows, and the forward values make no round trip: they replace the
-// transform value (leading parts) and 1/pivot (trailing parts) of their row.
-__global__ void __launch_bounds__(32)
+// Per row of 16 points: transform values, 1/pivot, and the off-diagonal of the row's
+// sweep; with the exchange between the sweeps the block's share.
+constexpr size_t spec_smem_df(int n) { return (size_t)n * (2 * 16 * 8 + 8); }
+constexpr size_t spec_smem_block(int n) { return spec_smem_df(n) + 2 * 32 * sizeof(dfl); }
+
+// Columns in shared memory, double-float: a block solves 16 consecutive spectral
+// points of the plane (n mp + m, padding columns included), a part of a point per
+// lane, warp 0 from the bottom wall and warp 1 from the top wall.  All loads are issued
+// before the first operation (cp.async), so a column costs one memory latency instead
+// of one per batch of rows, and the forward values make no round trip: their leading
+// parts replace the transform values of their row and their trailing parts its
+// pivots.  The back substitution's factors are prefetched to L2 and come in three
+// register batches.  Bound by the latency of the operations in a row's chain at the
+// few warps that the columns leave room for, so the sweeps run in whole batches without
+// branches, which the compiler overlaps: 89 instructions per row and warp, and 65.5
+// us at 256x193x256, against 111 and 101.6 with a guard per row (both parts of a point
+// in one lane, packed: 91.3; with the factors in shared memory too, two thirds of the
+// columns, and each part normalised by itself: 100.8).  A sweep by its own code with
+// constant strides: 78 instructions, but twice the code, 73 us, and 15.2 against 10.2
+// us at 64x65x64.
+__global__ void __launch_bounds__(64)
     k_spec_df_smem(cplx<float>* __restrict__ spec, SpecDF f, Geo g, float sc, bool neumann, bool skip_mean) {
   extern __shared__ __align__(16) unsigned char sp_smem[];
+  __shared__ dfl xch[2][32];
   const int n = g.nyc, tw = n / 2;
-  float2* rr = reinterpret_cast<float2*>(sp_smem);   // [n][16]
-  float2* iv = rr + (size_t)n * 16;                  // [n][16]
-  float2* cc = iv + (size_t)n * 16;                  // [n][16]
-  float2* ee = cc + (size_t)n * 16;                  // [2][n]: a, c
-  const int t = threadIdx.x, half = t >> 4, q = t & 15;
+  float* rr = reinterpret_cast<float*>(sp_smem);                    // [n][32]
+  float* iv = rr + (size_t)n * 32;                                  // [n][32]
+  float2* ee = reinterpret_cast<float2*>(iv + (size_t)n * 32);      // [n]
+  const int half = threadIdx.x >> 5, t = threadIdx.x & 31, q = t >> 1;
   const size_t P = (size_t)g.nz * g.mp, p0 = (size_t)blockIdx.x * 16;
-  const int most = max(tw, n - 1 - tw);              // rows of the longer sweep (the upper one: one more at most)
-  const int per = sp_group_rows(most);
+  const int rows = half ? n - 1 - tw : tw, j0 = half ? n - 1 : 0, dj = half ? -1 : 1;
   {
-    // copy e of a pair of rows (step i of both sweeps): 8 16-byte copies per row and array
-    const int c = t & 7, h = (t >> 3) & 1, arr = t >> 4;
+    // two rows at a time, 8 16-byte copies per row and array
+    const int c = t & 7, arr = (t >> 3) & 1;
     const char* src = arr ? reinterpret_cast<const char*>(f.inv + p0) : reinterpret_cast<const char*>(spec + p0);
     char* dst = reinterpret_cast<char*>(arr ? iv : rr);
-    for (int gr = 0; gr < 4; ++gr) {
-      const int i1 = min(most, (gr + 1) * per);
-      for (int i = gr * per; i < i1; ++i) {
-        const int j = h ? n - 1 - i : i;
-        if (h ? j > tw : j < tw) sp_cp_async16(dst + (size_t)j * 128 + 16 * c, src + (size_t)j * P * 8 + 16 * c);
-      }
-      if (gr == 3 && h == 0) sp_cp_async16(dst + (size_t)tw * 128 + 16 * c, src + (size_t)tw * P * 8 + 16 * c);
-      sp_commit();
+    for (int i = t >> 4; i < rows; i += 2) {
+      const int j = j0 + i * dj;
+      sp_cp_async16(dst + (size_t)j * 128 + 16 * c, src + (size_t)j * P * 8 + 16 * c);
     }
-    const char* cs = reinterpret_cast<const char*>(f.cpr + p0);
-    for (int i = most - 1 - arr; i >= 0; i -= 2) {   // two steps at a time, from the middle
-      const int j = h ? n - 1 - i : i;
-      if (h ? j > tw : j < tw) sp_cp_async16(reinterpret_cast<char*>(cc) + (size_t)j * 128 + 16 * c, cs + (size_t)j * P * 8 + 16 * c);
-    }
-    sp_commit();
+    if (half == 0 && t < 16) sp_cp_async16(dst + (size_t)tw * 128 + 16 * c, src + (size_t)tw * P * 8 + 16 * c);
   }
-  for (int j = t; j < n; j += 32) {
-    ee[j] = f.a[j];
-    ee[n + j] = f.c[j];
+  for (int i = t; i < rows; i += 32) {
+    const int j = j0 + i * dj;
+    ee[j] = (half ? f.c : f.a)[j];
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(f.cpr + p0 + (size_t)j * P));   // the back substitution's factors
   }
-  __syncwarp();
-  const int rows = half ? n - 1 - tw : tw, j0 = half ? n - 1 : 0, dj = half ? -1 : 1;
-  const int s16 = 16 * dj;
-  float2 *pr = rr + j0 * 16 + q, *pi = iv + j0 * 16 + q;
-  const float2* po = ee + (half ? n : 0) + j0;
-  const bool pin = neumann && half == 0 && p0 + q == 0;
-  df2 d{f2(0.f), f2(0.f)};
-  for (int i = 0; i < most; i += kSpRows) {
-    if (i % per == 0) {
-      sp_wait_group(i / per);
-      __syncwarp();   // every lane's copies of the group
-    }
-    if (i + kSpRows <= rows) {
-      float2 r[kSpRows], v[kSpRows], o[kSpRows];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();   // every lane's copies
+  const int s32 = 32 * dj, s16 = 16 * dj;
+  float *pr = rr + j0 * 32 + t, *pl = iv + j0 * 32 + t;
+  const float2 *pi = reinterpret_cast<const float2*>(iv) + j0 * 16 + q, *po = ee + j0;
+  if (neumann && half == 0 && p0 + q == 0) pr[0] = 0.f;
+  dfl d{0.f, 0.f};
+  // three batches under way: one in the chain, the next one's products, and the loads
+  // of the one after; whole batches only, so that a batch is one straight piece of code
+  constexpr int CH = 4;
+  const int nb = rows / CH;
+  if (nb) {
+    float r[CH];
+    float2 v[CH], o[CH];
+    dfl x[CH], y[CH];
+    auto load = [&](int b) {
+      const int i = CH * min(b, nb - 1);
 #pragma unroll
-      for (int u = 0; u < kSpRows; ++u) {
-        r[u] = pr[u * s16];
-        v[u] = pi[u * s16];
-        o[u] = po[u * dj];
+      for (int u = 0; u < CH; ++u) {
+        r[u] = pr[(i + u) * s32];
+        v[u] = pi[(i + u) * s16];
+        o[u] = po[(i + u) * dj];
       }
-      if (pin && i == 0) r[0] = f2(0.f);
+    };
+    auto products = [&]() {
 #pragma unroll
-      for (int u = 0; u < kSpRows; ++u) {
-        d = df2_mul(df2_sub_mul(r[u], dfl{o[u].x, o[u].y}, d), dfl{v[u].x, v[u].y});
-        pr[u * s16] = d.h;
-        pi[u * s16] = d.l;
+      for (int u = 0; u < CH; ++u) {
+        x[u] = sp_scaled(r[u], v[u]);
+        y[u] = df_mul(dfl{-o[u].x, -o[u].y}, dfl{v[u].x, v[u].y});
       }
-    } else {
-      for (int u = 0; u < kSpRows && i + u < rows; ++u) {
-        const float2 r = pin && i + u == 0 ? f2(0.f) : pr[u * s16], v = pi[u * s16], o = po[u * dj];
-        d = df2_mul(df2_sub_mul(r, dfl{o.x, o.y}, d), dfl{v.x, v.y});
-        pr[u * s16] = d.h;
-        pi[u * s16] = d.l;
+    };
+    load(0);
+    products();
+    load(1);
+    for (int b = 0; b < nb; ++b) {
+      __syncwarp();   // a point's two lanes have read the pivots that this batch overwrites
+#pragma unroll
+      for (int u = 0; u < CH; ++u) {
+        d = df_add_mul(x[u], y[u], d);
+        pr[(CH * b + u) * s32] = d.h;
+        pl[(CH * b + u) * s32] = d.l;
       }
+      products();
+      load(b + 2);
     }
-    pr += kSpRows * s16;
-    pi += kSpRows * s16;
-    po += kSpRows * dj;
   }
-  sp_wait<0>();
-  __syncwarp();
-  // the middle row, by the lower lanes; both halves go on from its solution
-  const df2 du{make_float2(__shfl_down_sync(0xffffffffu, d.h.x, 16), __shfl_down_sync(0xffffffffu, d.h.y, 16)),
-               make_float2(__shfl_down_sync(0xffffffffu, d.l.x, 16), __shfl_down_sync(0xffffffffu, d.l.y, 16))};
-  const bool store = (p0 + q) % g.mp < (size_t)g.mh && !(skip_mean && p0 + q == 0);
-  float2* out = reinterpret_cast<float2*>(spec + p0) + q;
-  df2 x;
-  {
-    const float2 r = rr[tw * 16 + q], v = iv[tw * 16 + q], a = ee[tw], c = ee[n + tw];
-    x = df2_mul(df2_sub_mul(df2_sub_mul(r, dfl{a.x, a.y}, d), dfl{c.x, c.y}, du), dfl{v.x, v.y});
-    if (store && half == 0) out[(size_t)tw * P] = __fmul2_rn(x.h, f2(sc));
-    x.h = make_float2(__shfl_sync(0xffffffffu, x.h.x, q), __shfl_sync(0xffffffffu, x.h.y, q));
-    x.l = make_float2(__shfl_sync(0xffffffffu, x.l.x, q), __shfl_sync(0xffffffffu, x.l.y, q));
+  for (int i = CH * nb; i < rows; ++i) {
+    const float2 v = pi[i * s16];
+    d = sp_forward(pr[i * s32], v, po[i * dj], d);
+    __syncwarp();
+    pr[i * s32] = d.h;
+    pl[i * s32] = d.l;
   }
-  // back substitution, away from the middle
+  // back substitution, away from the middle: its factors in three register batches
   const int jl = half ? tw + 1 : tw - 1;   // the last row eliminated
-  const float2 *bh = rr + jl * 16 + q, *bl = iv + jl * 16 + q, *bc = cc + jl * 16 + q;
-  float2* po2 = out + (ptrdiff_t)jl * (ptrdiff_t)P;
+  const float2* bc = f.cpr + p0 + q + (ptrdiff_t)jl * (ptrdiff_t)P;
   const ptrdiff_t step = -(ptrdiff_t)dj * (ptrdiff_t)P;
-  int i = rows;
-  for (; i >= kSpRows; i -= kSpRows) {
-    float2 h[kSpRows], l[kSpRows], c[kSpRows];
+  constexpr int CB = 8;
+  auto load_b = [&](int b, float2 (&c)[CB]) {   // batch b (past the end: the last row again)
 #pragma unroll
-    for (int u = 0; u < kSpRows; ++u) {
-      h[u] = bh[-u * s16];
-      l[u] = bl[-u * s16];
-      c[u] = bc[-u * s16];
-    }
+    for (int u = 0; u < CB; ++u) c[u] = __ldg(bc + min(b * CB + u, rows - 1) * step);
+  };
+  float2 cA[CB], cB[CB], cC[CB];
+  load_b(0, cA);
+  load_b(1, cB);
+  load_b(2, cC);
+  if (half) xch[0][t] = d;
+  __syncthreads();
+  const bool store = (p0 + q) % g.mp < (size_t)g.mh && !(skip_mean && p0 + q == 0);
+  float* out = reinterpret_cast<float*>(spec + p0) + t;
+  if (!half) {
+    const float2 v = reinterpret_cast<const float2*>(iv)[tw * 16 + q], a = f.a[tw], c = f.c[tw];
+    const dfl x = sp_middle(rr[tw * 32 + t], v, a, c, d, xch[0][t]);
+    if (store) out[2 * (size_t)tw * P] = __fmul_rn(x.h, sc);
+    xch[1][t] = x;
+  }
+  __syncthreads();
+  dfl x = xch[1][t];
+  const float *bh = rr + jl * 32 + t, *bl = iv + jl * 32 + t;
+  out += 2 * (ptrdiff_t)jl * (ptrdiff_t)P;
+  const int nc = rows / CB;
+  for (int b = 0; b < nc; ++b) {
 #pragma unroll
-    for (int u = 0; u < kSpRows; ++u) {
-      x = df2_sub_mul(df2{h[u], l[u]}, dfl{c[u].x, c[u].y}, x);
-      if (store) *po2 = __fmul2_rn(x.h, f2(sc));
-      po2 += step;
+    for (int u = 0; u < CB; ++u) {
+      x = df_add_mul(dfl{bh[-u * s32], bl[-u * s32]}, dfl{-cA[u].x, -cA[u].y}, x);
+      if (store) *out = __fmul_rn(x.h, sc);
+      out += 2 * step;
     }
-    bh -= kSpRows * s16;
-    bl -= kSpRows * s16;
-    bc -= kSpRows * s16;
+    bh -= CB * s32;
+    bl -= CB * s32;
+#pragma unroll
+    for (int u = 0; u < CB; ++u) {
+      cA[u] = cB[u];
+      cB[u] = cC[u];
+    }
+    load_b(b + 3, cC);
   }
-  for (; i > 0; --i) {
-    x = df2_sub_mul(df2{*bh, *bl}, dfl{bc->x, bc->y}, x);
-    if (store) *po2 = __fmul2_rn(x.h, f2(sc));
-    po2 += step;
-    bh -= s16;
-    bl -= s16;
-    bc -= s16;
-  }
+#pragma unroll
+  for (int u = 0; u < CB; ++u)
+    if (nc * CB + u < rows) {
+      x = df_add_mul(dfl{bh[-u * s32], bl[-u * s32]}, dfl{-cA[u].x, -cA[u].y}, x);
+      if (store) *out = __fmul_rn(x.h, sc);
+      out += 2 * step;
+    }
 }
 
 // The same, streamed: 32 points per block, warp 0 from the bottom wall and warp 1
 // from the top wall; rows come in double-buffered batches and the forward values
-// go through dscr.  For columns too long to keep enough blocks on an SM.
+// go through dscr.  For columns too long to keep enough blocks on an SM; bound by
+// memory (256x193x256: 73.8 us, 5.8 TB/s of its own traffic).
 __global__ void __launch_bounds__(64)
     k_spec_df_stream(cplx<float>* __restrict__ spec, float4* __restrict__ dscr, SpecDF f, Geo g, float sc,
                      bool neumann, bool skip_mean) {
@@ -1043,7 +1070,7 @@ __global__ void __launch_bounds__(64)
     for (int u = 0; u < kSpRows; ++u)
       if (i + u < rows) {
         const float2 o = __ldg(po + u * dj);
-        d = df2_mul(df2_sub_mul(pin && i + u == 0 ? f2(0.f) : r[u], dfl{o.x, o.y}, d), dfl{v[u].x, v[u].y});
+        d = sp_forward(pin && i + u == 0 ? f2(0.f) : r[u], v[u], o, d);
         pd[u * sP] = make_float4(d.h.x, d.h.y, d.l.x, d.l.y);
       }
     po += kSpRows * dj;
@@ -1067,7 +1094,7 @@ __global__ void __launch_bounds__(64)
   float2* out = reinterpret_cast<float2*>(spec) + p;
   if (!half) {
     const float2 r = out[(size_t)tw * P], v = f.inv[p + (size_t)tw * P], a = f.a[tw], c = f.c[tw];
-    const df2 x = df2_mul(df2_sub_mul(df2_sub_mul(r, dfl{a.x, a.y}, d), dfl{c.x, c.y}, xch[0][q]), dfl{v.x, v.y});
+    const df2 x = sp_middle(r, v, a, c, d, xch[0][q]);
     if (store) out[(size_t)tw * P] = __fmul2_rn(x.h, f2(sc));
     xch[1][q] = x;
   }
@@ -1091,7 +1118,7 @@ __global__ void __launch_bounds__(64)
 #pragma unroll
     for (int u = 0; u < kSpRows; ++u)
       if (i - u > 0) {
-        x = df2_sub_mul(df2{make_float2(dd[u].x, dd[u].y), make_float2(dd[u].z, dd[u].w)}, dfl{c[u].x, c[u].y}, x);
+        x = df2_add_mul(df2{make_float2(dd[u].x, dd[u].y), make_float2(dd[u].z, dd[u].w)}, dfl{-c[u].x, -c[u].y}, x);
         if (store) out[-u * sP] = __fmul2_rn(x.h, f2(sc));
       }
     out -= kSpRows * sP;
@@ -1332,23 +1359,31 @@ __global__ void __launch_bounds__(256) k_spec_mean(cplx<T>* __restrict__ spec, c
   }
 }
 
-// Columns in shared memory (launch code 16) or streamed (32); 0 and the other
-// codes: in shared memory where all blocks are resident at once.  There the solve
-// is one column's latency, on one wave: 13.2 against 15.2 us at 64x65x64 (19.6
-// streamed one-sided), 17.4 against 27.6 at 128x97x128, 29.0 against 58.4 at
-// 64x257x64.  Over more waves the few warps that the columns leave room for lose to
-// the bandwidth of many streams, and so they do beside other cases' kernels
-// (ensembles, whose waves add up, take the streamed form): 100.8 against 74.1 us at 256x193x256 (5.5 TB/s;
-// 105.3 one-sided, scalar), 136 against 91 at 128x385x128.
-double spec_smem_waves(const Geo& g) {
+// Blocks of the column kernel that an SM holds, and their waves.
+static int spec_smem_per_sm(const Geo& g) {
   constexpr size_t kMost = 227 * 1024;
-  const size_t need = spec_smem_df(g.nyc);
-  int dev = 0, sms = 0;
-  if (need > kMost || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return 1e30;
-  const size_t per_sm = kMost / (need + 1024);   // 1 KB per block is the system's
-  return (double)g.nz * g.mp / 16 / ((double)sms * (per_sm < 1 ? 1 : per_sm < 32 ? per_sm : 32));
+  const size_t need = spec_smem_block(g.nyc);
+  return need > kMost ? 0 : (int)std::min<size_t>(32, std::max<size_t>(1, kMost / (need + 1024)));   // 1 KB the system's
+}
+double spec_smem_waves(const Geo& g) {
+  const int per_sm = spec_smem_per_sm(g);
+  return per_sm ? (double)g.nz * g.mp / 16 / ((double)fft_sms() * per_sm) : 1e30;
+}
+
+// Columns in shared memory (launch code 16) or streamed (32); 0 and the other codes:
+// in shared memory where an SM holds four blocks or more (up to 214 rows), or where two
+// waves do it.  Pressure solve, in shared memory against streamed: 10.2 and 14.3 us
+// at 64x65x64, 14.8 and 27.1 at 128x97x128, 65.5 and 73.8 at 256x193x256, 206 and 247
+// at 512x193x512 (4 per SM); 48.9 and 88.9 at 128x385x128 (2 per SM, 1.9 waves), 58.4
+// and 107.9 at 128x513x64.  With fewer columns on an SM over more waves their bandwidth
+// falls behind that of many streams, and so does the step: 94.8 and 96.9 at 256x257x256
+// (a step of 512x257x256 6372 and 6338), 174.7 and 142.1 at 256x385x256, 1106 and 962
+// at 1024x385x512.  Beside other cases' kernels the streamed form wins (ensembles,
+// whose waves add up, take it: eight 128x97x128 cases 7811 and 7353 us).
+static bool spec_in_smem(const Geo& g) {
+  const int per_sm = spec_smem_per_sm(g);
+  if (g.lc_spec == 16 || g.lc_spec == 32) return g.lc_spec == 16 && per_sm > 0;
+  return per_sm >= 4 || spec_smem_waves(g) <= 2.0;
 }
 
 template <typename T>
@@ -1365,10 +1400,11 @@ cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f
   if (e != cudaSuccess) return e;
   const unsigned n16 = (unsigned)((size_t)g.nz * g.mp / 16);   // nz a multiple of 4, mp of 8
   const size_t need = spec_smem_df(g.nyc);
-  if (g.lc_spec == 16 ? need <= 227 * 1024 : g.lc_spec != 32 && spec_smem_waves(g) <= 1.0) {
-    if (need > 48 * 1024) e = cudaFuncSetAttribute(k_spec_df_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+  if (spec_in_smem(g)) {
+    if (spec_smem_block(g.nyc) > 48 * 1024)
+      e = cudaFuncSetAttribute(k_spec_df_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (e != cudaSuccess) return e;
-    k_spec_df_smem<<<n16, 32, need, s>>>(spec, f, g, (float)scale, neumann, mean != nullptr);
+    k_spec_df_smem<<<n16, 64, need, s>>>(spec, f, g, (float)scale, neumann, mean != nullptr);
   } else {
     k_spec_df_stream<<<n16 / 2, 64, 0, s>>>(spec, reinterpret_cast<float4*>(dscr), f, g, (float)scale, neumann,
                                             mean != nullptr);
@@ -1759,6 +1795,7 @@ cudaError_t launch_periodic_conv(const ConvArgs<T>& a, const Geo& g, cudaStream_
 
 template cudaError_t launch_periodic_conv<double>(const ConvArgs<double>&, const Geo&, cudaStream_t);
 template cudaError_t launch_periodic_conv<float>(const ConvArgs<float>&, const Geo&, cudaStream_t);
+
 
 template cudaError_t launch_fft_x_fwd<double, double>(PoissonSrc, const double*, const double*, const double*,
                                                       const double*, const double*, const double*, double,

@@ -42,18 +42,19 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   return df_fast_two_sum(p, e);
 }
 
-// r - a * b with r a float and a, b df.
-__device__ __forceinline__ dfl df_sub_mul(float r, dfl a, dfl b) {
-  const dfl p = df_mul(a, b);
-  const dfl s = df_two_sum(r, -p.h);
-  return df_two_sum(s.h, __fsub_rn(s.l, p.l));   // s.h may have cancelled: full TwoSum
-}
-
-// x - a * b with x, a, b df.
-__device__ __forceinline__ dfl df_sub_mul(dfl x, dfl a, dfl b) {
-  const dfl p = df_mul(a, b);
-  const dfl s = df_two_sum(x.h, -p.h);
-  return df_two_sum(s.h, __fadd_rn(s.l, __fsub_rn(x.l, p.l)));
+// x + a * b as one step of a recurrence in b: the product's trailing part is not
+// normalised before the sum, and the sum once, by FastTwoSum.  Error about 2^-47 (|x| +
+// |a b|), as with the parts normalised one by one; after a cancellation what FastTwoSum
+// drops is a rounding of the trailing part, 2^-48 of the operands.  Eight dependent
+// operations from b to the result's leading part, against 23.
+__device__ __forceinline__ dfl df_add_mul(dfl x, dfl a, dfl b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, e);
+  e = __fmaf_rn(a.l, b.h, e);
+  const dfl s = df_two_sum(x.h, p);
+  const float lo = __fadd_rn(s.l, __fadd_rn(x.l, e)), h = __fadd_rn(s.h, lo);
+  return {h, __fsub_rn(lo, __fsub_rn(h, s.h))};
 }
 
 // x + d + f with x, d df and f a float; renormalised with TwoSum because the
@@ -119,15 +120,14 @@ __device__ __forceinline__ df2 df2_mul(dfl b, df2 a) {
   const float2 s = __fadd2_rn(p, e);
   return {s, sub2(e, sub2(s, p))};
 }
-__device__ __forceinline__ df2 df2_sub_mul(float2 r, dfl a, df2 b) {
-  const df2 p = df2_mul(a, b);
-  const df2 s = df2_two_sum(r, __fmul2_rn(p.h, f2(-1.f)));
-  return df2_two_sum(s.h, sub2(s.l, p.l));
-}
-__device__ __forceinline__ df2 df2_sub_mul(df2 x, dfl a, df2 b) {
-  const df2 p = df2_mul(a, b);
-  const df2 s = df2_two_sum(x.h, __fmul2_rn(p.h, f2(-1.f)));
-  return df2_two_sum(s.h, __fadd2_rn(s.l, sub2(x.l, p.l)));
+__device__ __forceinline__ df2 df2_add_mul(df2 x, dfl a, df2 b) {
+  const float2 ah = f2(a.h), p = __fmul2_rn(ah, b.h);
+  float2 e = __ffma2_rn(ah, b.h, __fmul2_rn(p, f2(-1.f)));
+  e = __ffma2_rn(ah, b.l, e);
+  e = __ffma2_rn(f2(a.l), b.h, e);
+  const df2 s = df2_two_sum(x.h, p);
+  const float2 lo = __fadd2_rn(s.l, __fadd2_rn(x.l, e)), h = __fadd2_rn(s.h, lo);
+  return {h, sub2(lo, sub2(h, s.h))};
 }
 
 // Host-side split of a double into a df pair (hi = nearest float).
