@@ -13,7 +13,6 @@
 // no normalisation and the real ones a factor 2; the spectral solve multiplies by
 // 1/(2 Nx Nz).
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "pnp_common.cuh"
@@ -482,17 +481,10 @@ __global__ void __launch_bounds__(256) k_fft_x_inv_reg(PoissonDst dst, const cpl
   });
 }
 
-// SMs of the present device; asked of the runtime once per device, since a transform's
-// launch rule needs it on every call: an FP64 Poisson solve of 32x33x32, bound by its
-// launches' host time, 21.4-23.5 -> 19.5-20.8 us over three runs each in turn.
 static int fft_sms() {
-  static std::atomic<int> known[64];
   int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  const bool kept = dev >= 0 && dev < 64;
-  if (kept && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (kept) known[dev].store(sms, std::memory_order_relaxed);
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
   return sms;
 }
 
