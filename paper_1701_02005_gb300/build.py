@@ -6,6 +6,7 @@ the shared library against the static CUDA runtime.  Output:
 """
 from __future__ import annotations
 
+import glob
 import os
 import shutil
 import subprocess
@@ -44,7 +45,7 @@ def _newer(target, deps):
 
 def build_library(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, h) for h in ("pnp_common.cuh", "pnp_mixed.cuh", "pnp_wall.cuh")] + [os.path.join(INCLUDE, "pnp.h")]
+    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [os.path.join(INCLUDE, "pnp.h")]
     exe = nvcc()
     objs = []
     jobs = []
