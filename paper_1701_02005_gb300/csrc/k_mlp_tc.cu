@@ -22,14 +22,16 @@
 // epilogue covers accumulator columns 0-63, then 64-127; each half is handed to
 // the issuing warp through an mbarrier as soon as it is staged, so that the next
 // layer's first K steps run under the second half of the epilogue.  Waits are
-// bounded: on a timeout a kernel records PNP_ERR_TIMEOUT, waits once more
-// (bounded) for its MMAs and copies, frees its tensor memory and returns.
+// bounded: on a timeout a kernel records PNP_ERR_TIMEOUT; in every case the threads
+// that issued MMAs and copies wait (bounded) until these have completed before the
+// kernel frees its tensor memory and returns (pnp_mlpflow.cuh).
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cstdint>
 
 #include "pnp_common.cuh"
+#include "pnp_mlpflow.cuh"
 #include "pnp_wall.cuh"
 
 namespace pnp {
@@ -219,6 +221,7 @@ struct NetSmem {
   float red[4 * 8];
   unsigned long long ready[2];   // a half of the A tile is staged (one arrival per epilogue warp)
   unsigned long long done;       // the layer's MMAs have completed
+  unsigned long long drained;    // all MMAs have (used once)
   uint32_t slot;
 };
 
@@ -294,6 +297,7 @@ __device__ __forceinline__ uint32_t net_setup(NetSmem& s, uint32_t ncols, const 
     mbar_init(&s.ready[0], kEpiWarps);
     mbar_init(&s.ready[1], kEpiWarps);
     mbar_init(&s.done, 1);
+    mbar_init(&s.drained, 1);
   }
   const uint4* src = reinterpret_cast<const uint4*>(wimg);
   uint4* dst = reinterpret_cast<uint4*>(s.w);
@@ -312,36 +316,40 @@ __device__ __forceinline__ uint32_t net_setup(NetSmem& s, uint32_t ncols, const 
   return s.slot;
 }
 
-// A forward layer's MMAs: halves of K as they are handed over (the first layer's
-// K of 48 at once).  False when a wait ran out.
-__device__ __forceinline__ bool issue_forward(NetSmem& s, int l, uint32_t dcol, unsigned phase) {
-  const uint32_t id = idesc_bf16(kTcRows, layer_np(l), false, false);
-  const Operand a = k_major(s.a, kTcRows), b = k_major(s.w + img_off(l), layer_np(l));
-  if (!mbar_wait_tc(&s.ready[0], phase)) return false;
-  if (l == 0 && !mbar_wait_tc(&s.ready[1], phase)) return false;
-  fence_after();
-  const int mid = l == 0 ? kInPad / 16 : kMlpHidden / 32, end = layer_kp(l) / 16;
-  mma_steps(dcol, a, b, id, 0, mid, false);
-  if (l > 0) {
-    if (!mbar_wait_tc(&s.ready[1], phase)) return false;
-    fence_after();
-    mma_steps(dcol, a, b, id, mid, end, true);
-  }
-  mma_commit(&s.done);
-  return true;
+// The MMA thread's operations (pnp_mlpflow.cuh).  Layer l's accumulators: two column
+// blocks by turns, or (TRAIN) a block each for the first three layers and one that
+// layer 4, the output and the data gradients share.
+__device__ __forceinline__ bool drain_mmas(unsigned long long* bar) {
+  mma_commit(bar);
+  return mbar_wait_tc(bar, 0);
 }
 
-// da = dz W: dz from `a` (the A tile, or the output layer's), W^T by reading the
-// forward image with K along its rows.
-__device__ __forceinline__ bool issue_backward(NetSmem& s, int l, uint32_t dcol, unsigned phase) {
-  if (!mbar_wait_tc(&s.ready[0], phase) || !mbar_wait_tc(&s.ready[1], phase)) return false;
-  fence_after();
-  const bool out = l == kMlpLayers - 1;
-  mma_steps(dcol, k_major(out ? s.dz5 : s.a, kTcRows), mn_major(s.w + img_off(l), layer_np(l)),
-            idesc_bf16(kTcRows, kMlpHidden, false, true), 0, layer_np(l) / 16, false);
-  mma_commit(&s.done);
-  return true;
-}
+template <bool TRAIN>
+struct NetOps {
+  NetSmem& s;
+  uint32_t tmem;
+  __device__ uint32_t dcol(int l) const { return tmem + (TRAIN ? min(l, 3) : l & 1) * kMlpHidden; }
+  __device__ bool ready(int h, unsigned phase) {
+    if (!mbar_wait_tc(&s.ready[h], phase)) return false;
+    fence_after();
+    return true;
+  }
+  // z = a W^T, half h of K (the first layer's 48 at once)
+  __device__ void forward(int l, int h) {
+    const int mid = l == 0 ? kInPad / 16 : kMlpHidden / 32, end = layer_kp(l) / 16;
+    mma_steps(dcol(l), k_major(s.a, kTcRows), k_major(s.w + img_off(l), layer_np(l)),
+              idesc_bf16(kTcRows, layer_np(l), false, false), h ? mid : 0, h ? end : mid, h != 0);
+  }
+  // da = dz W: dz from the A tile or the output layer's, W^T by reading the forward
+  // image with K along its rows
+  __device__ void backward(int l) {
+    const bool out = l == kMlpLayers - 1;
+    mma_steps(dcol(3), k_major(out ? s.dz5 : s.a, kTcRows), mn_major(s.w + img_off(l), layer_np(l)),
+              idesc_bf16(kTcRows, kMlpHidden, false, true), 0, layer_np(l) / 16, false);
+  }
+  __device__ void commit() { mma_commit(&s.done); }
+  __device__ bool drain() { return drain_mmas(&s.drained); }
+};
 
 // 16 accumulator columns + bias as pairs
 __device__ __forceinline__ float2 z_pair(const float (&v)[16], const float* bias, int i) {
@@ -350,13 +358,10 @@ __device__ __forceinline__ float2 z_pair(const float (&v)[16], const float* bias
 
 constexpr float kInferClip = 6.0f;
 
-// what a kernel does once a wait has run out: record it and give the MMAs one
-// more bounded wait before the tensor memory is freed
-__device__ __forceinline__ void net_end(NetSmem& s, uint32_t tmem, uint32_t ncols, bool ok, unsigned phase, int* err) {
-  if (!ok) {
-    atomicExch(err, PNP_ERR_TIMEOUT);
-    mbar_wait_tc(&s.done, phase);
-  }
+// records a wait that ran out; the MMAs are drained, so the tensor memory can go
+// once every warp's reads of it are done
+__device__ __forceinline__ void net_end(uint32_t tmem, uint32_t ncols, bool ok, int* err) {
+  if (!ok) atomicExch(err, PNP_ERR_TIMEOUT);
   fence_before();
   __syncthreads();
   if (threadIdx.x < 32) tmem_dealloc(tmem, ncols);
@@ -391,10 +396,10 @@ __global__ void __launch_bounds__(kNetThreads, 1) k_mlp_infer_tc(const float* __
   unsigned phase = 0;
   bool ok = true;
   if (warp == kEpiWarps) {
-    if ((tid & 31) == 0)
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x)
-        for (int l = 0; l < kMlpLayers && ok; ++l, phase ^= 1u)
-          ok = issue_forward(s, l, tmem + (l & 1) * kMlpHidden, phase);
+    if ((tid & 31) == 0) {
+      NetOps<false> o{s, tmem};
+      ok = flow_network<kMlpLayers, false>(o, blockIdx.x, ntiles, gridDim.x);
+    }
     __syncwarp();
   } else {
     const int grp = warp & 3, quarter = warp >> 2, r = 32 * grp + (tid & 31);
@@ -447,7 +452,7 @@ __global__ void __launch_bounds__(kNetThreads, 1) k_mlp_infer_tc(const float* __
       }
     }
   }
-  net_end(s, tmem, kCols, ok, phase, err);
+  net_end(tmem, kCols, ok, err);
 }
 
 // Training, the rows' part: forward through all layers, the loss and its
@@ -482,12 +487,10 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   unsigned phase = 0;
   bool ok = true;
   if (warp == kEpiWarps) {
-    if ((tid & 31) == 0)
-      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        for (int l = 0; l < kMlpLayers && ok; ++l, phase ^= 1u)
-          ok = issue_forward(s, l, tmem + (l < 4 ? l * kMlpHidden : last), phase);
-        for (int l = kMlpLayers - 1; l > 0 && ok; --l, phase ^= 1u) ok = issue_backward(s, l, tmem + last, phase);
-      }
+    if ((tid & 31) == 0) {
+      NetOps<true> o{s, tmem};
+      ok = flow_network<kMlpLayers, true>(o, blockIdx.x, ntiles, gridDim.x);
+    }
     __syncwarp();
   } else {
     const int grp = warp & 3, quarter = warp >> 2, r = 32 * grp + (tid & 31);
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
   }
   __syncthreads();
   if (tid < 6) lpart[(size_t)blockIdx.x * 8 + tid] = (s.red[tid] + s.red[8 + tid]) + (s.red[16 + tid] + s.red[24 + tid]);
-  net_end(s, tmem, kCols, ok, phase, err);
+  net_end(tmem, kCols, ok, err);
 }
 
 // Weight gradients: one CTA takes every splits[l]-th tile of layer l and
@@ -642,8 +645,27 @@ struct WgSmem {
   unsigned char b[kWgStages][kTileBytes + 16 * kTcRows * 2];
   unsigned long long full[kWgStages], empty[kWgStages];   // ring slots
   unsigned long long sum[2], free[2];                     // TMEM blocks: a sum is complete / has been read
+  unsigned long long drained;                             // all MMAs have completed (used once)
   uint32_t slot;
   int bad;
+};
+
+// The MMA thread's operations (pnp_mlpflow.cuh).
+struct WgOps {
+  WgSmem& s;
+  uint32_t tmem, id;
+  __device__ bool freed(int block, unsigned phase) { return mbar_wait_tc(&s.free[block], phase); }
+  __device__ bool full(int q, unsigned phase) {
+    if (!mbar_wait_tc(&s.full[q], phase)) return false;
+    fence_after();
+    return true;
+  }
+  __device__ void product(int q, int block, bool acc) {
+    mma_steps(tmem + block * 256, mn_major(s.a[q], kTcRows), mn_major(s.b[q], kTcRows), id, 0, kTcRows / 16, acc);
+  }
+  __device__ void commit_slot(int q) { mma_commit(&s.empty[q]); }
+  __device__ void commit_sum(int block) { mma_commit(&s.sum[block]); }
+  __device__ bool drain() { return drain_mmas(&s.drained); }
 };
 
 __global__ void __launch_bounds__(kWgThreads, 1)
@@ -669,6 +691,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
       mbar_init(&s.sum[q], 1);
       mbar_init(&s.free[q], 4);
     }
+    mbar_init(&s.drained, 1);
     s.bad = 0;
   }
   if (!out && l > 0)   // columns 128 .. 143 of B: ones in column 128
@@ -737,21 +760,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     // thread unless a wait ran out)
     for (int m = n > kWgStages ? n - kWgStages : 0; m < n; ++m) mbar_wait_tc(&s.full[m % kWgStages], (m / kWgStages) & 1);
   } else if (tid == 160) {
-    const uint32_t id = idesc_bf16(kTcRows, N, true, true);
-    for (int n = 0; n < ntl; ++n) {
-      const int q = n % kWgStages, g = n / kWgRun;
-      if (n % kWgRun == 0 && g >= 2 && !(ok = mbar_wait_tc(&s.free[g & 1], ((g >> 1) - 1) & 1))) break;
-      if (!(ok = mbar_wait_tc(&s.full[q], (n / kWgStages) & 1))) break;
-      fence_after();
-      mma_steps(tmem + (g & 1) * 256, mn_major(s.a[q], kTcRows), mn_major(s.b[q], kTcRows), id, 0, kTcRows / 16,
-                n % kWgRun != 0);
-      mma_commit(&s.empty[q]);
-      if (n % kWgRun == kWgRun - 1 || n == ntl - 1) mma_commit(&s.sum[g & 1]);
-    }
-    if (!ok) {   // the MMAs issued so far have completed before the tensor memory is freed
-      mma_commit(&s.sum[0]);
-      mbar_wait_tc(&s.sum[0], 0);
-    }
+    WgOps o{s, tmem, idesc_bf16(kTcRows, N, true, true)};
+    ok = flow_wgrad<kWgStages, kWgRun>(o, ntl);
   }
   if (!ok) s.bad = 1;
   __syncthreads();
