@@ -6,12 +6,23 @@
 // divergence (Eq. (2)).  All sums are FP64 with a fixed reduction order
 // (deterministic across runs for a given grid).
 #include <algorithm>
+#include <mutex>
 
 #include "pnp_common.cuh"
 #include "pnp_df.cuh"
 #include "pnp_mixed.cuh"
 
 namespace pnp {
+
+cudaError_t allow_smem(const void* kern, size_t smem) {
+  if (smem <= 40 * 1024) return cudaSuccess;   // 48 KB with the kernel's static part need no asking
+  static std::mutex one;
+  const std::lock_guard<std::mutex> hold(one);
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, kern);
+  if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
 
 // SplitMix64 (Steele, Lea & Flood 2014) used as a counter-based generator:
 // output n of the stream seeded by `seed` is mix(seed + (n + 1) * gamma).

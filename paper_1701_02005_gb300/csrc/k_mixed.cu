@@ -401,12 +401,10 @@ cudaError_t launch_mixed_cn(const Fields<float>& f, const Shadows& sh, const Mix
       a.f[0] = CnFamily{reinterpret_cast<const float*>(f.rcp), sh.cp, sh.cpL, R.dC_p + (size_t)l * g.nyc, ion, g.nyc};
       a.f[1] = CnFamily{reinterpret_cast<const float*>(f.rcm), sh.cm, sh.cmL, R.dC_m + (size_t)l * g.nyc, ion, g.nyc};
       const size_t smem = cn_tile_smem(g.nyc, 2);
-      if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_cn_tile<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-      }
+      cudaError_t e = allow_smem(k_cn_tile<2>, smem);
+      if (e != cudaSuccess) return e;
       k_cn_tile<2><<<dim3((unsigned)(P / 32), 2), blk, smem, s>>>(a);
-      const cudaError_t e = cudaGetLastError();
+      e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
     if (parts & kCnVelocity) {
@@ -416,10 +414,8 @@ cudaError_t launch_mixed_cn(const Fields<float>& f, const Shadows& sh, const Mix
       a.f[1] = CnFamily{f.rv + P, f.v + P, nullptr, nullptr, face, g.nyc - 1};   // interior faces 1 .. nyc-1
       a.f[2] = CnFamily{f.rw, f.w, nullptr, nullptr, cell, g.nyc};
       const size_t smem = cn_tile_smem(g.nyc, 1);
-      if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_cn_tile<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-      }
+      const cudaError_t e = allow_smem(k_cn_tile<1>, smem);
+      if (e != cudaSuccess) return e;
       k_cn_tile<1><<<dim3((unsigned)(P / 32), 3), blk, smem, s>>>(a);
       return cudaGetLastError();
     }

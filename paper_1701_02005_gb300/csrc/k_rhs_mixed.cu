@@ -972,7 +972,7 @@ cudaError_t launch_mixed_rhs(const Fields<float>& f, const Shadows& sh, const Mi
       using G = decltype(geo);
       const size_t smem = G::bytes(jc);
       if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = allow_smem(kern, smem);
       if (e != cudaSuccess) return e;
       const dim3 grd((unsigned)(g.nz / tzb), (unsigned)((g.nyc + jc - 1) / jc));
       kern<<<grd, dim3(g.nx, tzb), smem, s>>>(*maps, f, rp, rm, sh, R, g, m, cf, jc, err, fz);
@@ -988,10 +988,8 @@ cudaError_t launch_mixed_rhs(const Fields<float>& f, const Shadows& sh, const Mi
   auto go = [&](auto kern, int bx, int bz, int cz, bool hsm) {
     const dim3 grd((unsigned)(g.nx / bx), (unsigned)(g.nz / (bz * cz)), (unsigned)((g.nyc + jc - 1) / jc));
     const size_t smem = sizeof(float) * (rhs_tile_floats(bx, bz, cz, hsm) + (size_t)kPlaneLd * jc);
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<grd, dim3(bx, bz), smem, s>>>(f, rp, rm, sh, R, g, m, cf, jc, fz);
     return cudaGetLastError();
   };

@@ -529,10 +529,8 @@ cudaError_t launch_fft_x_fwd(PoissonSrc kind, const TV* u, const TV* v, const TV
     auto go = [&](auto kern, int G, size_t (*smem_of)(int)) {
       const int nrows = g.nyc * g.nz, rows = fx_rows(G, nrows, sizeof(T) == 8);
       const size_t smem = smem_of(rows);
-      if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-      }
+      const cudaError_t e = allow_smem(kern, smem);
+      if (e != cudaSuccess) return e;
       kern<<<(nrows + rows - 1) / rows, dim3(G, rows), smem, s>>>(a, g, m, spec, tw_half, tw_post);
       return cudaGetLastError();
     };
@@ -549,10 +547,8 @@ cudaError_t launch_fft_x_fwd(PoissonSrc kind, const TV* u, const TV* v, const TV
   dim3 blk, grd;
   size_t smem;
   fft_x_shape<T>(g, blk, grd, smem);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_fft_x_fwd<T, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_fft_x_fwd<T, TV>, smem);
+  if (e != cudaSuccess) return e;
   k_fft_x_fwd<T, TV><<<grd, blk, smem, s>>>(a, g, m, spec, tw_half, tw_post);
   return cudaGetLastError();
 }
@@ -618,10 +614,8 @@ cudaError_t launch_fft_x_inv(PoissonDst dst, const cplx<T>* spec, const Geo& g, 
     auto go = [&](auto kern, int G, size_t (*smem_of)(int)) {
       const int nrows = g.nyc * g.nz, rows = fx_rows(G, nrows, sizeof(T) == 8);
       const size_t smem = smem_of(rows);
-      if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-      }
+      const cudaError_t e = allow_smem(kern, smem);
+      if (e != cudaSuccess) return e;
       kern<<<(nrows + rows - 1) / rows, dim3(G, rows), smem, s>>>(dst, spec, g, m, tw_half, tw_post, V, out, plane_add,
                                                                   cell_add);
       return cudaGetLastError();
@@ -639,10 +633,8 @@ cudaError_t launch_fft_x_inv(PoissonDst dst, const cplx<T>* spec, const Geo& g, 
   dim3 blk, grd;
   size_t smem;
   fft_x_shape<T>(g, blk, grd, smem);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_fft_x_inv<T, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_fft_x_inv<T, TO>, smem);
+  if (e != cudaSuccess) return e;
   k_fft_x_inv<T, TO><<<grd, blk, smem, s>>>(dst, spec, g, m, tw_half, tw_post, V, out, plane_add, cell_add);
   return cudaGetLastError();
 }
@@ -754,10 +746,8 @@ cudaError_t launch_fft_z_reg(cplx<T>* spec, const cplx<T>* tw, const Geo& g, boo
   const dim3 grd = DENSE ? dim3((unsigned)((g.mh * g.nyc + TM - 1) / TM))
                          : dim3((unsigned)((g.mh + TM - 1) / TM), (unsigned)g.nyc);
   auto go = [&](auto kern) {
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<grd, dim3(TM, G), smem, s>>>(spec, tw, g);
     return cudaGetLastError();
   };
@@ -788,10 +778,8 @@ cudaError_t launch_fft_z(cplx<T>* spec, const cplx<T>* tw_z, const Geo& g, bool 
   dim3 blk(TM, ty, 1);
   dim3 grd((g.mh + TM - 1) / TM, g.nyc, 1);
   const size_t smem = (size_t)2 * TM * (g.nz + 1) * sizeof(cplx<T>);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_fft_z<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(k_fft_z<T>, smem);
+  if (e != cudaSuccess) return e;
   k_fft_z<T><<<grd, blk, smem, s>>>(spec, tw_z, g, inverse);
   return cudaGetLastError();
 }
@@ -1401,8 +1389,7 @@ cudaError_t launch_spec_thomas_df(cplx<float>* spec, void* dscr, const SpecDF& f
   const unsigned n16 = (unsigned)((size_t)g.nz * g.mp / 16);   // nz a multiple of 4, mp of 8
   const size_t need = spec_smem_df(g.nyc);
   if (spec_in_smem(g)) {
-    if (spec_smem_block(g.nyc) > 48 * 1024)
-      e = cudaFuncSetAttribute(k_spec_df_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    e = allow_smem(k_spec_df_smem, need);
     if (e != cudaSuccess) return e;
     k_spec_df_smem<<<n16, 64, need, s>>>(spec, f, g, (float)scale, neumann, mean != nullptr);
   } else {
@@ -1626,10 +1613,8 @@ cudaError_t launch_periodic(const PeriodicArgs<T>& a, const Geo& g, bool zdir, c
   for (int q = 0; q < a.nfam; ++q) maxp = a.f[q].nplanes > maxp ? a.f[q].nplanes : maxp;
   const int nblk = zdir ? maxp * (g.nx / L) : maxp * g.nz / L;
   auto kern = zdir ? k_periodic<T, true> : k_periodic<T, false>;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
   kern<<<dim3((unsigned)nblk, (unsigned)a.nfam, 1), 128, smem, s>>>(a, g, L);
   return cudaGetLastError();
 }
@@ -1772,10 +1757,8 @@ cudaError_t launch_periodic_conv(const ConvArgs<T>& a, const Geo& g, cudaStream_
   const size_t smem = (size_t)kConvRing * g.nx * sizeof(T);
   const dim3 grd((unsigned)maxp, (unsigned)a.nfam);
   auto go = [&](auto kern) {
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<grd, nt, smem, s>>>(a, g);
     return cudaGetLastError();
   };

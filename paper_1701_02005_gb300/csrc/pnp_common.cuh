@@ -139,6 +139,17 @@ __host__ __device__ inline size_t cidx(int j, int k, int i, int nz, int nx) {
 }
 
 // ---- launchers (host functions; all asynchronous on stream) ----
+// Lets a kernel have smem bytes of dynamic shared memory.  The attribute belongs to the
+// function and not to a launch, a stream or a thread, so where the size depends on the
+// grid it must never go down: a context on a smaller grid that lowered it between
+// another thread's setting and its launch would have that launch refused.  One thread
+// at a time reads it and raises it where smem is more.
+cudaError_t allow_smem(const void* kern, size_t smem);
+template <typename... A>
+cudaError_t allow_smem(void (*kern)(A...), size_t smem) {
+  return allow_smem(reinterpret_cast<const void*>(kern), smem);
+}
+
 template <typename TV>
 cudaError_t launch_rhs(const Fields<TV>& f, const Geo& g, const Metrics& m, const Phys& ph,
                        const Stage& st, cudaStream_t s);
