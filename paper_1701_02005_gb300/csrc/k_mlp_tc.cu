@@ -862,12 +862,15 @@ cudaError_t mlp_infer_tc(const MlpBufs& b, const float* X, int B, float* Y, cuda
   return cudaGetLastError();
 }
 
-// How many CTAs share each layer's tiles: the SMs in proportion to the bytes per
-// tile (44, 64, 64, 64 and 36 KB of 272), at most one per tile; a layer's slice of
-// the partial sums per CTA.
-WgPlan mlp_wgrad_plan(int ntiles) {
+// How many CTAs share each layer's tiles: one wave of the SMs (a CTA takes one by its
+// shared and tensor memory), in proportion to the bytes per tile (44, 64, 64, 64 and 36
+// KB of 272), at most one per tile; a layer's slice of the partial sums per CTA.
+WgPlan mlp_wgrad_plan(int ntiles, int sms) {
   const MlpDims d = mlp_dims();
-  const int share[kMlpLayers] = {24, 36, 36, 36, 20};   // of the 152 SMs: one wave
+  constexpr int full[kMlpLayers] = {24, 36, 36, 36, 20};
+  static_assert(full[0] + full[1] + full[2] + full[3] + full[4] == kWgCtas, "shares of kWgCtas");
+  int share[kMlpLayers];
+  share_ctas(full, kWgCtas, sms, share);
   WgPlan p{};
   size_t off = 0;
   for (int l = 0; l < kMlpLayers; ++l) {
@@ -894,7 +897,7 @@ cudaError_t mlp_train_tc(const MlpBufs& b, const float* X, const float* T, int B
   k_mlp_train_tc<<<(unsigned)grid, kNetThreads, sizeof(NetSmem), s>>>(
       X, T, B, aligned16(X) ? 1 : 0, b.wimg, d, b.param, b.in_shift, b.in_scale, b.out_shift, b.out_scale, b.skip_out,
       b.skip_in, b.atiles, b.dztiles, b.lpart, b.err);
-  const WgPlan plan = mlp_wgrad_plan(ntiles);
+  const WgPlan plan = mlp_wgrad_plan(ntiles, sms);
   int nblk = 0;
   for (int l = 0; l < kMlpLayers; ++l) nblk += plan.splits[l];
   k_mlp_wgrad_tc<<<(unsigned)nblk, kWgThreads, sizeof(WgSmem), s>>>(b.atiles, b.dztiles, ntiles, plan, b.partial, b.err);

@@ -2368,7 +2368,7 @@ size_t mlp_carve(pnp_mlp* m, char* base, int max_batch) {
   const int ntiles = (max_batch - 1) / 128 + 1;
   b.atiles = bp.take<unsigned char>(ntiles * kATileBytes);
   b.dztiles = bp.take<unsigned char>(ntiles * kDzTileBytes);
-  b.partial = bp.take<float>(mlp_wgrad_plan(ntiles).total);
+  b.partial = bp.take<float>(mlp_wgrad_plan(ntiles, kWgCtas).total);
   b.lpart = bp.take<float>(8 * kMlpMaxRowCtas);
   b.loss = bp.take<float>(1);
   b.in_shift = bp.take<float>(kMlpIn);

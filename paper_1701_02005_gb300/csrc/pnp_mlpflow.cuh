@@ -1,8 +1,8 @@
 // The order in which the MMA thread of a network kernel (k_mlp_tc.cu) waits and
 // issues, as templates over the operations themselves, so that the host can run it
-// with waits that run out.
+// with waits that run out; and how the weight gradients' CTAs are shared out.
 //
-// Both end in o.drain(), whatever ended the loop: it commits everything the thread has
+// Both flows end in o.drain(), whatever ended the loop: it commits everything the thread has
 // issued to a barrier that nothing else uses and waits for that (bounded).  A barrier
 // of the loop cannot serve: a layer whose second half was never handed over has MMAs
 // that no commit covers, and the phase of a barrier whose last use is unknown may be
@@ -59,6 +59,25 @@ PNP_FLOW bool flow_wgrad(Ops& o, int ntl) {
     if (n % RUN == RUN - 1 || n == ntl - 1) o.commit_sum(g & 1);
   }
   return o.drain() && ok;
+}
+
+// How `ctas` CTAs, one per SM, share the layers' tiles, given the shares of `full` of
+// them: in proportion, at least one each, and no layer more than of `full` (the partial
+// sums are laid out for those).
+template <int N>
+inline void share_ctas(const int (&of_full)[N], int full, int ctas, int (&out)[N]) {
+  ctas = ctas < full ? ctas : full;
+  int left = ctas;
+  for (int l = 0; l < N; ++l) {
+    out[l] = of_full[l] * ctas / full;
+    if (out[l] < 1) out[l] = 1;
+    left -= out[l];
+  }
+  for (int l = 0; left > 0; l = (l + 1) % N)
+    if (out[l] < of_full[l]) {
+      ++out[l];
+      --left;
+    }
 }
 
 }  // namespace pnp

@@ -89,7 +89,8 @@ struct WgPlan {
   int splits[kMlpLayers];
   size_t len[kMlpLayers], off[kMlpLayers], total;
 };
-WgPlan mlp_wgrad_plan(int ntiles);
+constexpr int kWgCtas = 152;   // at most, all layers together: what the partial sums are laid out for
+WgPlan mlp_wgrad_plan(int ntiles, int sms);
 
 // Buffers of one MLP (all device pointers, carved by the host code).
 struct MlpBufs {

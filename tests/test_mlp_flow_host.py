@@ -1,7 +1,7 @@
 """The MMA threads' order of waits and issues (pnp_mlpflow.cuh), run on the host: the
 parities of a run in which every wait succeeds, and, with each wait in turn running
 out, that nothing issued is still under way when the kernel goes on to free its
-tensor memory."""
+tensor memory; and how the weight gradients' CTAs are shared out over fewer SMs."""
 import os
 import shutil
 import subprocess
@@ -98,12 +98,37 @@ int main() {
 """
 
 
-def test_nothing_issued_is_left_under_way(tmp_path):
+SHARES = r"""
+#include <cstdio>
+#include "pnp_mlpflow.cuh"
+
+int main() {
+  const int full[5] = {24, 36, 36, 36, 20};
+  for (int sms = 0; sms <= 200; ++sms) {
+    int s[5], sum = 0, most = sms < 152 ? sms : 152;
+    pnp::share_ctas(full, 152, sms, s);
+    for (int l = 0; l < 5; ++l) {
+      sum += s[l];
+      const double part = full[l] * most / 152.0;
+      if (s[l] < 1 || s[l] > full[l] || (most >= 5 && (s[l] < part - 2 || s[l] > part + 2)) ||
+          (sms >= 152 && s[l] != full[l]))
+        return std::printf("%d SMs: layer %d gets %d\n", sms, l, s[l]), 1;
+    }
+    // one wave, and no SM without a CTA; below eight SMs the layers' ones alone can exceed it
+    if (most >= 8 ? sum != most : sum > 8) return std::printf("%d SMs: %d CTAs\n", sms, sum), 1;
+  }
+  std::puts("ok");
+}
+"""
+
+
+@pytest.mark.parametrize("program", [PROGRAM, SHARES], ids=["order", "shares"])
+def test_host_side_of_the_network_kernels(program, tmp_path):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
     src, exe = tmp_path / "flow.cpp", tmp_path / "flow"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
