@@ -343,16 +343,17 @@ int pnp_selftest_wait_timeout(pnp_ctx* ctx, double limit_s);
 int pnp_fp64_peak(pnp_ctx* ctx, double* flops_out);
 
 /* Autotuner (no counterpart in the paper; launch-shape selection for GB300):
- * times candidate launch codes of the stencil (FP64: block x-extent 16/32/64/128
- * of 128 threads; mixed: 16 one-cell tiles, 32 / 64 packed two-cell tiles
- * 32 / 64 cells wide, 128 TMA rows), the
- * wall-normal CN sweeps (32 = mixed
- * shared-memory line tiles, else 64/128/256 threads per block), the spectral
- * y-solves (mixed: 16 = columns in shared memory, 32 = streamed; other codes
- * choose by the grid) and the
- * z-transform (8..64 threads per column; mixed: 64 = stage-by-stage kernel,
- * else register FFT) on this context's grid with CUDA events and keeps the
- * fastest; then re-checks each choice, one code at a time, on the time of
+ * times candidate launch codes of the stencil (FP64: 16 a cell per thread in blocks
+ * of 16 cells in x, other codes the march over y-planes on tiles as wide as Nx
+ * allows, or, below 32 cells in x, a cell per thread in blocks of 32/64/128; mixed:
+ * 16 one-cell tiles, 32 / 64 packed two-cell tiles 32 / 64 cells wide, 128 TMA
+ * rows), the wall-normal CN sweeps (32 = mixed shared-memory line tiles, else
+ * 64/128/256 threads per block), the spectral y-solves (mixed: 16 = columns in
+ * shared memory, 32 = streamed, other codes choose by the grid; FP64: streamed
+ * whatever the code) and the z-transform (8..64 threads per column; 64 =
+ * stage-by-stage kernel, else register FFT for Nz of 16 to 512) on this context's
+ * grid with CUDA events and keeps the fastest of the codes that stand for different
+ * launches there; then re-checks each choice, one code at a time, on the time of
  * whole steps of size dt (pnp_step from a Poisson-Boltzmann initial state),
  * since launch shapes interact inside a step.  cfg_out[4] receives the choice
  * (same order as pnp_set_launch_config), ms_out[4] (optional) the best time of

@@ -1366,8 +1366,12 @@ double spec_smem_waves(const Geo& g) {
 // and 107.9 at 128x513x64.  With fewer columns on an SM over more waves their bandwidth
 // falls behind that of many streams, and so does the step: 94.8 and 96.9 at 256x257x256
 // (a step of 512x257x256 6372 and 6338), 174.7 and 142.1 at 256x385x256, 1106 and 962
-// at 1024x385x512.  Beside other cases' kernels the streamed form wins (ensembles,
-// whose waves add up, take it: eight 128x97x128 cases 7811 and 7353 us).
+// at 1024x385x512.  Beside other cases' kernels the streamed form wins with the
+// fused CN elimination: ensembles, whose waves add up, take it in the place of this
+// choice above one wave (a step of four 64x65x64 and four 128x97x128 cases 1473 and 1384
+// us, of 24 each 9159 and 8529).  A code of 16 stays there, the autotuner's too: with
+// the CN line tiles that it picks on these grids the columns in shared memory win
+// (1434 and 1533 us, 8997 and 9502).
 static bool spec_in_smem(const Geo& g) {
   const int per_sm = spec_smem_per_sm(g);
   if (g.lc_spec == 16 || g.lc_spec == 32) return g.lc_spec == 16 && per_sm > 0;

@@ -2070,11 +2070,22 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
   const int reps = 3;
   float best[4] = {1e30f, 1e30f, 1e30f, 1e30f};
   int pick[4] = {32, 128, 64, 32};
-  // 1: stencil block shape
+  // the codes that stand for different launches on this grid, per site
+  const bool fp64 = c->precision == PNP_FP64;
+  std::vector<int> cands[4] = {{}, {32, 64, 128, 256}, {16, 32}, {}};
   for (int bx : {32, 64, 128, 16}) {
-    // FP64: block x-extents; mixed: 128 = TMA rows (when available), 64 / 32 / 16 = cp.async tiles
-    if (c->precision == PNP_FP64 && bx > 2 * c->g.nx && bx != 32) continue;
-    if (c->precision == PNP_MIXED && bx == 128 && !c->rhs_maps_ok) continue;
+    // FP64: 16 = a cell per thread, else the march (from 32 cells in x; below, block
+    // x-extents); mixed: 128 = TMA rows (when available), 64 / 32 / 16 = cp.async tiles
+    if (fp64 && (c->g.nx >= 32 ? bx != 32 && bx != 16 : bx > 2 * c->g.nx && bx != 32)) continue;
+    if (!fp64 && bx == 128 && !c->rhs_maps_ok) continue;
+    cands[0].push_back(bx);
+  }
+  if (fp64) cands[2] = {64};   // streamed whatever the code
+  const bool reg_z = c->g.nz >= 16 && c->g.nz <= 512;   // 64 = stage by stage, the other codes all register transforms
+  for (int ty : {8, 16, 32, 64})
+    if (reg_z ? ty == 32 || (ty == 64 && ty <= c->g.nz / 4) : ty == 8 || ty <= c->g.nz / 4) cands[3].push_back(ty);
+  // 1: stencil block shape
+  for (int bx : cands[0]) {
     c->g.lc_rhs_bx = bx;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64) launch_rhs<double>(fields<double>(c), c->g, metrics(c), c->ph, st, c->stream);
@@ -2085,7 +2096,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
   }
   c->g.lc_rhs_bx = pick[0];
   // 2: CN sweep block size
-  for (int T : {32, 64, 128, 256}) {   // mixed: 32 = shared-memory line tiles
+  for (int T : cands[1]) {   // mixed: 32 = shared-memory line tiles
     c->g.lc_cn = T;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64)
@@ -2099,7 +2110,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
   c->g.lc_cn = pick[1];
   // 3: spectral y-solve (columns in shared memory or streamed), 4: z-transform threads per column
   const double scale = 0.5 / ((double)c->g.nx * (double)c->g.nz);   // the forward x-transform's values are doubled
-  for (int T : {16, 32}) {   // (FP64 has the streamed form only)
+  for (int T : cands[2]) {
     c->g.lc_spec = T;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64)
@@ -2112,8 +2123,7 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
     if (t < best[2]) { best[2] = t; pick[2] = T; }
   }
   c->g.lc_spec = pick[2];
-  for (int ty : {8, 16, 32, 64}) {
-    if (ty > 8 && ty > c->g.nz / 4) continue;
+  for (int ty : cands[3]) {
     c->g.lc_fftz_ty = ty;
     float t = time_launches(c, [&] {
       if (c->precision == PNP_FP64)
@@ -2161,13 +2171,9 @@ int pnp_autotune(pnp_ctx* c, double dt, int* cfg_out, double* ms_out) {
       *f[i] = v;
     };
     float cur = step_ms();
-    const std::vector<int> cands[4] = {{32, 64, 128, 16}, {32, 64, 128, 256}, {16, 32}, {8, 16, 32, 64}};
     for (int i = 0; i < 4; ++i) {
       for (int v : cands[i]) {
         if (v == pick[i]) continue;
-        if (i == 0 && c->precision == PNP_FP64 && v > 2 * c->g.nx && v != 32) continue;
-        if (i == 0 && c->precision == PNP_MIXED && v == 128 && !c->rhs_maps_ok) continue;
-        if (i == 3 && v > 8 && v > c->g.nz / 4) continue;
         set(i, v);
         const float t = step_ms();
         if (t < 0.99f * cur) {

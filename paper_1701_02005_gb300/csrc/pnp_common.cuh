@@ -29,11 +29,13 @@ struct Geo {
   int mh, mp;            // nx/2 + 1 spectral columns, padded pitch
   double dx, dz, idx, idz;
   // launch shapes chosen by the autotuner (0 = built-in default)
-  int lc_rhs_bx;         // FP64 stencil: x-extent of the 128-thread blocks (16, 32, 64, 128);
+  int lc_rhs_bx;         // FP64 stencil: 16 = a cell per thread in blocks of 16 x 8, else the march over
+                         // planes (nx < 32: a cell per thread, the x-extent of 128-thread blocks);
                          // mixed stencil: 128 TMA rows, 64 / 32 packed-pair cp.async tiles 64 / 32
                          // cells wide, 16 one-cell tiles
   int lc_cn;             // threads per block of the wall-normal CN sweeps (mixed: 32 = shared-memory line tiles)
   int lc_spec;           // spectral y-solves (mixed): 16 = columns in shared memory, 32 = streamed, else by size
+                         // (FP64: streamed)
   int lc_fftz_ty;        // threads per column of the z-transform (cap)
 };
 
