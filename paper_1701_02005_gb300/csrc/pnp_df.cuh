@@ -46,7 +46,12 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
 // normalised before the sum, and the sum once, by FastTwoSum.  Error about 2^-47 (|x| +
 // |a b|), as with the parts normalised one by one; after a cancellation what FastTwoSum
 // drops is a rounding of the trailing part, 2^-48 of the operands.  Eight dependent
-// operations from b to the result's leading part, against 23.
+// operations from b to the result's leading part, against 23.  A whole elimination's rms
+// error against 80-bit arithmetic, relative to its column's largest value, with the
+// parts normalised one by one and so: 6.0e-15 and 5.4e-15 at 64 rows (1.3e-15 and
+// 1.2e-15 between Dirichlet walls), 3.3e-14 and 3.0e-14 at 192 (1.6e-15 and 2.0e-15),
+// 2.9e-13 both at 384: it goes either way, 1e-5 of the rounding of the FP32 solution
+// that is stored (8e-9).
 __device__ __forceinline__ dfl df_add_mul(dfl x, dfl a, dfl b) {
   const float p = __fmul_rn(a.h, b.h);
   float e = __fmaf_rn(a.h, b.h, -p);
@@ -108,15 +113,6 @@ __device__ __forceinline__ df2 df2_mul(df2 a, dfl b) {
   float2 e = __ffma2_rn(a.h, bh, __fmul2_rn(p, f2(-1.f)));
   e = __ffma2_rn(a.h, f2(b.l), e);
   e = __ffma2_rn(a.l, bh, e);
-  const float2 s = __fadd2_rn(p, e);
-  return {s, sub2(e, sub2(s, p))};
-}
-// b * a with b the first factor of df_mul (the order of the cross terms)
-__device__ __forceinline__ df2 df2_mul(dfl b, df2 a) {
-  const float2 bh = f2(b.h), p = __fmul2_rn(bh, a.h);
-  float2 e = __ffma2_rn(bh, a.h, __fmul2_rn(p, f2(-1.f)));
-  e = __ffma2_rn(bh, a.l, e);
-  e = __ffma2_rn(f2(b.l), a.h, e);
   const float2 s = __fadd2_rn(p, e);
   return {s, sub2(e, sub2(s, p))};
 }
