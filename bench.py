@@ -51,10 +51,16 @@ def cells(wl=WL):
 # (shape = the stencil's tuned launch code the capture ran with)
 # DRAM bytes (read + write) of all 45 launches of one step of that workload, from the
 # one-pass ncu capture summarised under profiles/ (cold cache: ncu flushes L2 before
-# each kernel), per cell-step, for the launch shapes the capture ran with
-STEP_NCU = {"mixed": {"bytes_per_cell_step": 839.6, "cells": 12582912, "shape": [64, 64, 32, 16],
-                     "note": "45 launches, 582 B read + at least 257 B written per cell-step (writes still in L2 "
+# each kernel), per cell-step, for the launches the capture ran: the 64-wide stencil tile
+# with the fused CN elimination, the y-solves' columns in shared memory, register transforms
+STEP_NCU = {"mixed": {"bytes_per_cell_step": 752.1, "cells": 12582912,
+                     "note": "45 launches, 548 B read + at least 204 B written per cell-step (writes still in L2 "
                              "at a kernel's end are not counted)"}}
+
+
+def step_ncu_launches(cfg, fused, columns):
+    """Whether a run's launch codes (None: the defaults) are the launches STEP_NCU was captured with."""
+    return fused and columns and (cfg is None or (cfg[0] == 64 and cfg[1] != 32 and cfg[3] != 64))
 
 # Algorithmic bytes per cell-step of the whole step (every input read once, every
 # output written once per phase; the phases the method's synchronisation points
@@ -66,23 +72,41 @@ NCU_TRAFFIC = {
     # mean of three consecutive launches (one per RK3 substage) of the stencil with
     # the fused CN forward elimination, launch code 0 / 64
     ("mixed", "rhs"): {"kernel": "k_rhs_mixed_tile<64, 4, 2, false, 2> (fused CN forward elimination)",
-                       "shape": (0, 64), "cells": 12582912, "bytes": 913655040},
+                       "shape": (0, 64), "cells": 12582912, "bytes": 912467200},
 }
 
 
-def site_cost(site, precision, launch_cfg=None, fused=True):
+def columns_in_smem(nx, ny, nz, code, sms=152):
+    """Whether the mixed y-solves keep their columns in shared memory: launch code 16
+    where a column block fits, 32 never, the others where an SM holds four blocks (264 B
+    a row) or two waves of blocks of 16 columns do all of a plane."""
+    need = 264 * (ny - 1) + 512
+    per_sm = 0 if need > 227 * 1024 else min(32, max(1, 227 * 1024 // (need + 1024)))
+    if code in (16, 32) or per_sm == 0:
+        return code == 16 and per_sm > 0
+    pitch = (nx // 2 + 1 + 7) // 8 * 8
+    return per_sm >= 4 or nz * pitch / 16 <= 2.0 * sms * per_sm
+
+
+def site_cost(site, precision, launch_cfg=None, fused=True, columns=False):
+    """Bytes and FP64-pipe instructions of a launch site per cell; columns: the mixed
+    y-solves with their columns in shared memory (columns_in_smem)."""
     half = (WL["nx"] // 2 + 1) / WL["nx"]
+    # mixed y-solves: value in and out and two df factors per spectral point; streamed
+    # ones also write and re-read the df forward values
+    solve = (32 if columns else 64) * half
     # mixed CN: the back substitution after the stencil's fused forward elimination
     # (the default) and the shared-memory line tiles (launch code 32) move 76 B per
     # cell (d in, state in and out); the unfused line kernels also write and re-read d (116 B)
     cn_tiled = fused or (launch_cfg is not None and launch_cfg[1] == 32)
     if precision == "fp64":
+        # FP64-pipe instructions as ncu counts them at Nx = Nz = 256 (summarised under profiles/)
         table = {
-            "rhs": (176, 220), "cn_thomas": (200, 20),
-            "p_fftx": (24 + 16 * half, 30), "p_fftz": (32 * half, 20), "p_thomas": (80 * half, 10 * half),
-            "p_ifftz": (32 * half, 20), "p_ifftx": (16 * half + 8, 22), "project": (72, 8),
-            "e_fftx": (16 + 16 * half, 24), "e_fftz": (32 * half, 20), "e_thomas": (80 * half, 10 * half),
-            "e_ifftz": (32 * half, 20), "e_ifftx": (16 * half + 8, 22),
+            "rhs": (176, 155), "cn_thomas": (200, 20),
+            "p_fftx": (24 + 16 * half, 19.1), "p_fftz": (32 * half, 11.2), "p_thomas": (80 * half, 4.3),
+            "p_ifftz": (32 * half, 11.2), "p_ifftx": (16 * half + 8, 12.9), "project": (72, 8),
+            "e_fftx": (16 + 16 * half, 15.1), "e_fftz": (32 * half, 11.2), "e_thomas": (80 * half, 4.3),
+            "e_ifftz": (32 * half, 11.2), "e_ifftx": (16 * half + 8, 13.9),
         }
     else:
         table = {
@@ -90,9 +114,9 @@ def site_cost(site, precision, launch_cfg=None, fused=True):
             # previous H (20 B) when zeta != 0 and the new H (20 B) except in the
             # last substage: 68, 88, 68 B over the three substages
             "rhs": (224 / 3, 0), "cn_thomas": (76 if cn_tiled else 116, 0),
-            "p_fftx": (12 + 8 * half, 0), "p_fftz": (16 * half, 0), "p_thomas": (64 * half, 0),
+            "p_fftx": (12 + 8 * half, 0), "p_fftz": (16 * half, 0), "p_thomas": (solve, 0),
             "p_ifftz": (16 * half, 0), "p_ifftx": (8 * half + 4, 0), "project": (36, 0),
-            "e_fftx": (8 + 8 * half, 0), "e_fftz": (16 * half, 0), "e_thomas": (64 * half, 0),
+            "e_fftx": (8 + 8 * half, 0), "e_fftz": (16 * half, 0), "e_thomas": (solve, 0),
             "e_ifftz": (16 * half, 0), "e_ifftx": (8 * half + 4, 0.25),
         }
     b, f = table[site]
@@ -1164,15 +1188,17 @@ def run_ours(args):
         pass
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     hbm_src = "MEASURED_PEAKS.json hbm_gbs (measured copy)" if "hbm_gbs" in peaks else "fallback 6800 GB/s"
+    columns = columns_in_smem(WL["nx"], WL["ny"], WL["nz"], launch_cfg[2] if launch_cfg else 0,
+                              torch.cuda.get_device_properties(local).multi_processor_count)
     sites = {}
     for k, v in per_launch.items():
-        cst = site_cost(k, pname, launch_cfg, not args.no_fusion)
+        cst = site_cost(k, pname, launch_cfg, not args.no_fusion, columns)
         d = v * 1e-3
         gbs = cst["bytes"] * n_cells / d / 1e9
         tf = 2.0 * cst["fp64_ops"] * n_cells / d / 1e12   # FP64 ops counted as FMA-equivalent flops
         sites[k] = {"ms": round(v, 4), "share": round(v / total, 4), "hbm_frac": round(gbs / hbm_peak, 4),
                     "fp64_frac": round(tf / (fp64_peak / 1e12), 4)}
-    cst = site_cost(dom, pname, launch_cfg, not args.no_fusion)
+    cst = site_cost(dom, pname, launch_cfg, not args.no_fusion, columns)
     dur = per_launch[dom] * 1e-3
     hbm_gbs = cst["bytes"] * n_cells / dur / 1e9
     alu_tf = 2.0 * cst["fp64_ops"] * n_cells / dur / 1e12
@@ -1201,7 +1227,7 @@ def run_ours(args):
     step_roof["frac_of_measured"] = step_roof["achieved_gbs"] / hbm_peak
     step_roof["frac_of_nominal"] = step_roof["achieved_gbs"] / NOMINAL_HBM_GBS
     sn = STEP_NCU.get(pname)
-    if sn and sn["cells"] == n_cells and (sn["shape"] is None or (launch_cfg and list(launch_cfg) == sn["shape"])):
+    if sn and sn["cells"] == n_cells and step_ncu_launches(launch_cfg, not args.no_fusion, columns):
         g_ncu = sn["bytes_per_cell_step"] * n_cells * K / t / 1e9
         step_roof.update({"ncu_bytes_per_cell_step": sn["bytes_per_cell_step"], "ncu_gbs": g_ncu,
                           "ncu_frac_of_measured": g_ncu / hbm_peak, "ncu_frac_of_nominal": g_ncu / NOMINAL_HBM_GBS,
