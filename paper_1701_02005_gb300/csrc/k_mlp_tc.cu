@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
 // tensor cores' FP32 sums are not rounded to nearest, so a sum of 256 rows (2e-7
 // of the gradient) goes on in registers (over all of a CTA's rows in TMEM the
 // error was 2e-6).  Per tile 64 KB are read for 4.2 MFLOP, so the copies bound
-// it: 5.5 TB/s.  Each CTA writes its sums to its own slice of `partial`.
+// it: 5.4 TB/s.  Each CTA writes its sums to its own slice of `partial`.
 constexpr int kWgStages = 3, kWgThreads = 192, kWgRun = 2;   // stages; threads; tiles per TMEM sum
 constexpr int kWgCols = kMlpHidden + 16;
 struct WgSmem {

@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(128) k_rhs(Fields<TV> f, Geo g, Metrics mt, Ph
 // serves u's z-flux and w's x-flux.  Factors 1/2 and 1/4 of the averages are part
 // of the (exactly scaled) constants, and all constants of a plane come from a
 // per-block table.  About 155 FP64 operations per cell (and 5 for the tile's
-// edges) against 235: 128x97x128, 0.96 -> 0.50 ms, the FP64 pipe 84% busy.  Wide
-// tiles for few x-edges: 0.60 ms at 64x2, 0.55 ms at 128x2 for one version.
+// edges) against 235: 128x97x128, 0.96 -> 0.50 ms, the FP64 pipe 79% busy.  The tiles
+// are as wide as Nx allows, for few x-edges.
 // ---------------------------------------------------------------------------
 struct MarchPlane {   // constants of plane j (face j and, suffix p, face j + 1)
   double idy4, idy2;                   // 1/(4 dy), 1/(2 dy)

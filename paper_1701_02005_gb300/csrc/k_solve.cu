@@ -25,11 +25,10 @@ namespace pnp {
 // Crank-Nicolson y-solves.  One thread per (i, k) line; lines are consecutive
 // in x so every plane access is coalesced.  The matrix I - s L_y is the same
 // for every line, so its elimination factors (a, c, m) come precomputed.
-// One launch for all five families: a small grid's families run side by side and a
-// step has three launches fewer, a large one's share one last wave; the velocities
-// and the ions one after the other before.  Three 32x33x32 contexts in turn 97 ->
-// 92 us a step, 128x97x128 2865 -> 2831.  Blocks of 128 lines: of 32 and 64 lines 97
-// and 93 us, though a context alone takes 174.5 a step with those and 176.4 with 128.
+// Bound by the latency of the sweeps on small grids and by memory on large ones.  One
+// launch for all five families: a small grid's run side by side, a large one's share
+// one last wave (three 32x33x32 contexts stepped in turn 97 -> 92 us a step, three of
+// 128x97x128 2865 -> 2831, against the velocities and the ions one after the other).
 // ---------------------------------------------------------------------------
 struct CnFam {
   double *q, *r;   // state and right-hand side at the family's first row
@@ -884,13 +883,9 @@ constexpr size_t spec_smem_block(int n) { return spec_smem_df(n) + 2 * 32 * size
 // parts replace the transform values of their row and their trailing parts its
 // pivots.  The back substitution's factors are prefetched to L2 and come in three
 // register batches.  Bound by the latency of the operations in a row's chain at the
-// few warps that the columns leave room for, so the sweeps run in whole batches without
-// branches, which the compiler overlaps: 89 instructions per row and warp, and 65.5
-// us at 256x193x256, against 111 and 101.6 with a guard per row (both parts of a point
-// in one lane, packed: 91.3; with the factors in shared memory too, two thirds of the
-// columns, and each part normalised by itself: 100.8).  A sweep by its own code with
-// constant strides: 78 instructions, but twice the code, 73 us, and 15.2 against 10.2
-// us at 64x65x64.
+// few warps that the columns leave room for, so a lane holds one part of a point and
+// the sweeps run in whole batches without branches, which the compiler overlaps: 89
+// instructions per row and warp.  256x193x256: 65.5 us, 73.8 streamed.
 __global__ void __launch_bounds__(64)
     k_spec_df_smem(cplx<float>* __restrict__ spec, SpecDF f, Geo g, float sc, bool neumann, bool skip_mean) {
   extern __shared__ __align__(16) unsigned char sp_smem[];
